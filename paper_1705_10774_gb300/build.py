@@ -29,7 +29,9 @@ SOURCES = [
 ]
 # floating-point flags of each precision code: FP64 without contraction
 # (parity with the oracle), FP32 with fast division and square root, FP64
-# with fused multiply-adds
+# with fused multiply-adds.  The ideal-MHD kernels write their fused
+# multiply-adds out, so that every tile shape rounds alike, and contract
+# nothing else.
 PREC_FLAGS = {0: ["-fmad=false"], 1: ["-ftz=true", "-prec-div=false", "-prec-sqrt=false"], 2: []}
 
 
@@ -50,7 +52,7 @@ def units(checked=False):
     for vid, t, tx, ty, nt, mb, prec, rs, ni in variants(checked):
         defs = ["-DV_ID=%d" % vid, "-DV_T=%s" % t, "-DV_TX=%d" % tx, "-DV_TY=%d" % ty, "-DV_NT=%d" % nt,
                 "-DV_MB=%d" % mb, "-DV_PREC=%d" % prec, "-DV_RS=%d" % rs, "-DV_NI=%d" % ni]
-        out.append(("dsp_variant.cu", "dsp_variant_%d.o" % vid, defs + PREC_FLAGS[prec]))
+        out.append(("dsp_variant.cu", "dsp_variant_%d.o" % vid, defs + PREC_FLAGS[prec] + ([] if ni or prec == 0 else ["-fmad=false"])))
     return out
 
 

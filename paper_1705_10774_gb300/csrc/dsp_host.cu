@@ -552,6 +552,25 @@ const KernelVariant *(*const kVariants[])() = {DSP_VARIANT_LIST(DSP_VARIANT_ENTR
 #undef DSP_VARIANT_ENTRY
 constexpr int kNumVariants = sizeof(kVariants) / sizeof(kVariants[0]);
 
+// SM time of one plane of one tile of a variant, relative to the other
+// variants of its form (measured on 256^3 cells in 32^3 patches: time of a
+// sweep over its tiles).  A patch's default variant is the one with the
+// smallest cost times its number of tiles, so that wide tiles serve patches
+// they divide and 16 x 8 tiles serve the small and the ragged ones.
+double tile_cost(const KernelVariant *v) {
+  if (v->nonideal || v->riemann) return 1.0;
+  switch (v->id) {
+    case 1: return 0.66;   // FP64, 8 x 8
+    case 3: return 0.60;   // FP64 with FMA, 8 x 8
+    case 4: return 1.17;   // FP64 with FMA, 16 x 12
+    case 6: return 1.40;   // FP32, 16 x 8, one block per SM
+    case 7: return 1.76;   // FP32, 32 x 8
+    case 8: return 1.94;   // FP32, 16 x 16
+    case 21: return 1.74;  // FP32, 24 x 8
+    default: return 1.0;   // 16 x 8
+  }
+}
+
 // Per-patch tiles and offsets, each patch tiled by its class's tile shape
 // tx[k] x ty[k] and z run tz[k]; false if some tile's owner table would not
 // fit the kernel's table.
@@ -908,10 +927,28 @@ extern "C" int dsp_create(const dsp_patch_desc *patches, int32_t npatch, const d
       for (int d = 0; d < 3; d++) cls_n[0][d] = sizes.back()[(size_t)d];
     }
   }
+  // the classes' default variants: the requested one, else the cheapest per
+  // patch among those of this form (the first where they tie)
+  const KernelVariant *varc[MAXCLS];
+  for (int k = 0; k < MAXCLS; k++) {
+    varc[k] = var;
+    if (prm->variant >= 0 || k >= ncls) continue;
+    double best = INFINITY;
+    for (int q = 0; q < kNumVariants; q++) {
+      const KernelVariant *v = kVariants[q]();
+      if (v->precision != prm->precision || v->riemann != prm->riemann || v->nonideal != nonideal) continue;
+      const double cost = tile_cost(v) * ((cls_n[k][0] + v->tx - 1) / v->tx) * ((cls_n[k][1] + v->ty - 1) / v->ty);
+      if (cost < best) {
+        best = cost;
+        varc[k] = v;
+      }
+    }
+  }
+  var = varc[0];
   int tzc[MAXCLS], txc[MAXCLS], tyc[MAXCLS];
   for (int k = 0; k < MAXCLS; k++) {
-    txc[k] = var->tx;
-    tyc[k] = var->ty;
+    txc[k] = varc[k]->tx;
+    tyc[k] = varc[k]->ty;
     tzc[k] = 0;
   }
   for (int i = 0; i < npatch; i++) tzc[cls[(size_t)i]] = std::max(tzc[cls[(size_t)i]], patches[i].n[2]);
@@ -947,7 +984,7 @@ extern "C" int dsp_create(const dsp_patch_desc *patches, int32_t npatch, const d
   c->cls = cls;
   c->ncls = ncls;
   for (int k = 0; k < MAXCLS; k++) {
-    c->var_cls[k] = var;
+    c->var_cls[k] = varc[k];
     c->tz_cls[k] = tzc[k];
     for (int dd = 0; dd < 3; dd++) c->cls_n[k][dd] = cls_n[k][dd];
   }

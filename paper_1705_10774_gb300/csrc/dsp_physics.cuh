@@ -43,6 +43,12 @@ struct FBits<float> {
   static __device__ __forceinline__ float to(I i) { return __int_as_float(i); }
   static constexpr I MAG = 0x7fffffff, INF = 0x7f800000;
 };
+// Bits of |a| from the value's two halves: masking the 64-bit pattern instead
+// is compiled to an FP64 absolute value, which takes an FP64-pipe slot.
+__device__ __forceinline__ long long mag_bits(double a) {
+  return ((long long)(__double2hiint(a) & 0x7fffffff) << 32) | (unsigned)__double2loint(a);
+}
+__device__ __forceinline__ int mag_bits(float a) { return __float_as_int(a) & 0x7fffffff; }
 // |a| (as fabs: the sign bit cleared, for every input); in FP32 the native
 // form, which the FP32 pipe folds into the operation that uses it
 template <typename T>
@@ -65,8 +71,8 @@ __device__ __forceinline__ bool tpos(T a) {
 template <typename T>
 __device__ __forceinline__ bool tneg(T a) {
   using B = FBits<T>;
-  const typename B::I i = B::of(a), m = i & B::MAG;
-  return i < 0 && m != 0 && m <= B::INF;
+  const typename B::I m = mag_bits(a);
+  return B::of(a) < 0 && m != 0 && m <= B::INF;
 }
 // min(a, b) for a, b >= +0 or NaN (as fmin: a NaN operand yields the other)
 template <typename T>
@@ -186,6 +192,25 @@ __device__ __forceinline__ T sqrt_k(T x) {
   }
 }
 
+// a b + c and c - a b: one rounding under kFast, else two; a / b: by the
+// reciprocal under kFast.
+template <typename T>
+__device__ __forceinline__ T madd(T a, T b, T c) {
+  if constexpr (!kFast) return a * b + c;
+  else if constexpr (sizeof(T) == 8) return fma(a, b, c);
+  else return fmaf(a, b, c);
+}
+template <typename T>
+__device__ __forceinline__ T nmadd(T a, T b, T c) {
+  if constexpr (!kFast) return c - a * b;
+  else return madd(-a, b, c);
+}
+template <typename T>
+__device__ __forceinline__ T quot(T a, T b) {
+  if constexpr (!kFast) return a / b;
+  else return a * rcp_k(b);
+}
+
 // Primitive state (rho, v, p, B) from conserved (rho, m, E) and the six faces.
 // With `floored`, *floored tells whether the pressure floor was taken.
 template <typename T>
@@ -256,6 +281,14 @@ __device__ __forceinline__ T signal_sum(const T W[8], T gamma) {
   return (tabs(W[VX]) + cx) + (tabs(W[VY]) + cy) + (tabs(W[VZ]) + cz);
 }
 
+// The value of the larger magnitude (NaN if either is).
+template <typename T>
+__device__ __forceinline__ T fmax_mag(T a, T b) {
+  using B = FBits<T>;
+  const typename B::I i = mag_bits(a), j = mag_bits(b);
+  return B::to(i > j ? i : j);
+}
+
 // Monotonised-central limited slope: zero when the one-sided differences
 // have opposite signs or one is zero, else the smallest of twice either and
 // their mean, with their sign.  The tests are on sign bits (the same result
@@ -264,9 +297,8 @@ template <typename T>
 __device__ __forceinline__ T mc(T dl, T dr) {
   using B = FBits<T>;
   const typename B::I a = B::of(dl), b = B::of(dr);
-  if ((a & B::MAG) == 0 || (b & B::MAG) == 0 || (a ^ b) < 0) return T(0);
-  if constexpr (kFast && sizeof(T) == 8) {
-    // the same value as 2 min(|dl|, |dr|, |dl + dr| / 4): the power-of-two
+  if constexpr (sizeof(T) == 8) {
+    // 2 min(|dl|, |dr|, |dl + dr| / 4): the power-of-two
     // scalings are exact, so they are done on the bit patterns with integer
     // operations, leaving one FP64 operation, dl + dr.  Both arms of each
     // select are integer: near the ends of the exponent range, x/4 of a
@@ -274,8 +306,10 @@ __device__ __forceinline__ T mc(T dl, T dr) {
     // rounded to nearest even (as the multiply would round it), 2x of a
     // subnormal x is its pattern shifted left, 2x of the largest binade is
     // infinity, and an infinity or NaN stays as it is.
-    const long long m = min(a & B::MAG, b & B::MAG);
-    const long long iq0 = __double_as_longlong(dl + dr) & B::MAG;
+    const long long ma = mag_bits(dl), mb = mag_bits(dr);
+    if (ma == 0 || mb == 0 || (a ^ b) < 0) return T(0);
+    const long long m = min(ma, mb);
+    const long long iq0 = mag_bits(dl + dr);
     const long long one = 1ll << 52;
     const int eq = (int)(iq0 >> 52);
     long long iq;
@@ -295,13 +329,11 @@ __device__ __forceinline__ T mc(T dl, T dr) {
     const int es = (int)(is >> 52);
     const long long i2 = es == 0 ? is << 1 : es < 2046 ? is + one : es == 2046 ? 0x7ff0000000000000ll : is;
     return __longlong_as_double(a < 0 ? i2 | (long long)0x8000000000000000ull : i2);
-  } else if constexpr (sizeof(T) == 4) {
+  } else {
     // FP32: the FP32 pipe's own minimum (the same value as the bit-pattern
     // minimum of non-negative values) and absolute-value modifiers
+    if ((a & B::MAG) == 0 || (b & B::MAG) == 0 || (a ^ b) < 0) return T(0);
     const T s = fminf(fminf(T(2) * fabsf(dl), T(2) * fabsf(dr)), T(0.5) * fabsf(dl + dr));
-    return a < 0 ? B::to(B::of(s) ^ ~B::MAG) : s;
-  } else {
-    const T s = tmin_nonneg(tmin_nonneg(T(2) * tabs(dl), T(2) * tabs(dr)), T(0.5) * tabs(dl + dr));
     return a < 0 ? B::to(B::of(s) ^ ~B::MAG) : s;
   }
 }
@@ -409,19 +441,19 @@ __device__ __forceinline__ void hlld(const T WL[8], const T WR[8], T gamma, T ig
     rho[a] = W[RHO]; u[a] = W[VX + D]; v[a] = W[VX + t1]; w[a] = W[VX + t2];
     by[a] = W[BX + t1]; bz[a] = W[BX + t2];
     const T p = W[PR];
-    const T v2 = u[a] * u[a] + v[a] * v[a] + w[a] * w[a];
-    const T B2 = bx * bx + by[a] * by[a] + bz[a] * bz[a];
-    E[a] = p * igm1 + h * rho[a] * v2 + h * B2;
-    PT[a] = p + h * B2;
-    vB[a] = u[a] * bx + v[a] * by[a] + w[a] * bz[a];
-    c[a] = cfast(gamma, T(1) / rho[a], p, bx, by[a], bz[a]);
+    const T v2 = madd(w[a], w[a], madd(v[a], v[a], u[a] * u[a]));
+    const T B2 = madd(bz[a], bz[a], madd(by[a], by[a], bx * bx));
+    E[a] = madd(h, B2, madd(h * rho[a], v2, p * igm1));
+    PT[a] = madd(h, B2, p);
+    vB[a] = madd(w[a], bz[a], madd(v[a], by[a], u[a] * bx));
+    c[a] = cfast(gamma, rcp_k(rho[a]), p, bx, by[a], bz[a]);
     Us[a][0] = rho[a]; Us[a][1] = rho[a] * u[a]; Us[a][2] = rho[a] * v[a]; Us[a][3] = rho[a] * w[a];
     Us[a][4] = E[a];
     Fs[a][0] = rho[a] * u[a];
-    Fs[a][1] = rho[a] * u[a] * u[a] + PT[a] - bx * bx;
-    Fs[a][2] = rho[a] * u[a] * v[a] - bx * by[a];
-    Fs[a][3] = rho[a] * u[a] * w[a] - bx * bz[a];
-    Fs[a][4] = (E[a] + PT[a]) * u[a] - bx * vB[a];
+    Fs[a][1] = nmadd(bx, bx, madd(rho[a] * u[a], u[a], PT[a]));
+    Fs[a][2] = nmadd(bx, by[a], rho[a] * u[a] * v[a]);
+    Fs[a][3] = nmadd(bx, bz[a], rho[a] * u[a] * w[a]);
+    Fs[a][4] = nmadd(bx, vB[a], (E[a] + PT[a]) * u[a]);
   }
   SL = tmin(u[0] - c[0], u[1] - c[1]);
   SR = tmax(u[0] + c[0], u[1] + c[1]);
@@ -435,63 +467,63 @@ __device__ __forceinline__ void hlld(const T WL[8], const T WR[8], T gamma, T ig
   } else {
     const T Sa[2] = {SL, SR};
     const T dl = (SL - u[0]) * rho[0], dr = (SR - u[1]) * rho[1];
-    const T iden = T(1) / (dr - dl);
-    const T SM = ((dr * u[1] - dl * u[0]) - PT[1] + PT[0]) * iden;
-    const T PTs = ((dr * PT[0] - dl * PT[1]) + dl * dr * (u[1] - u[0])) * iden;
+    const T iden = rcp_k(dr - dl);
+    const T SM = (nmadd(dl, u[0], dr * u[1]) - PT[1] + PT[0]) * iden;
+    const T PTs = madd(dl * dr, u[1] - u[0], nmadd(dl, PT[1], dr * PT[0])) * iden;
     T rs[2], vs[2], ws[2], bys[2], bzs[2], Es[2], sr[2];
 #pragma unroll
     for (int a = 0; a < 2; a++) {
-      const T su = Sa[a] - u[a];
-      rs[a] = rho[a] * su / (Sa[a] - SM);
-      const T den = rho[a] * su * (Sa[a] - SM) - bx * bx;
-      const T ref = rho[a] * su * su + bx * bx;
+      const T su = Sa[a] - u[a], sm = Sa[a] - SM;
+      rs[a] = quot(rho[a] * su, sm);
+      const T den = nmadd(bx, bx, rho[a] * su * sm);
+      const T ref = madd(bx, bx, rho[a] * su * su);
       if (tabs(den) <= T(1e-12) * ref) {
         vs[a] = v[a]; ws[a] = w[a]; bys[a] = by[a]; bzs[a] = bz[a];
       } else {
-        const T iv = T(1) / den;
+        const T iv = rcp_k(den);
         const T fv = bx * (SM - u[a]) * iv;
-        const T fb = (rho[a] * su * su - bx * bx) * iv;
-        vs[a] = v[a] - by[a] * fv;
-        ws[a] = w[a] - bz[a] * fv;
+        const T fb = nmadd(bx, bx, rho[a] * su * su) * iv;
+        vs[a] = nmadd(by[a], fv, v[a]);
+        ws[a] = nmadd(bz[a], fv, w[a]);
         bys[a] = by[a] * fb;
         bzs[a] = bz[a] * fb;
       }
-      const T vBs = SM * bx + vs[a] * bys[a] + ws[a] * bzs[a];
-      Es[a] = ((su * E[a] - PT[a] * u[a] + PTs * SM) + bx * (vB[a] - vBs)) / (Sa[a] - SM);
-      sr[a] = tsqrt(rs[a]);
+      const T vBs = madd(ws[a], bzs[a], madd(vs[a], bys[a], SM * bx));
+      Es[a] = quot(madd(bx, vB[a] - vBs, madd(PTs, SM, nmadd(PT[a], u[a], su * E[a]))), sm);
+      sr[a] = sqrt_k(rs[a]);
     }
     const T aB = tabs(bx);
-    const T SsL = SM - aB / sr[0], SsR = SM + aB / sr[1];
+    const T SsL = SM - quot(aB, sr[0]), SsR = SM + quot(aB, sr[1]);
     if (SsL >= T(0)) {
       const T Ust[5] = {rs[0], rs[0] * SM, rs[0] * vs[0], rs[0] * ws[0], Es[0]};
 #pragma unroll
-      for (int k = 0; k < 5; k++) Fr[k] = Fs[0][k] + SL * (Ust[k] - Us[0][k]);
+      for (int k = 0; k < 5; k++) Fr[k] = madd(SL, Ust[k] - Us[0][k], Fs[0][k]);
     } else if (SsR <= T(0)) {
       const T Ust[5] = {rs[1], rs[1] * SM, rs[1] * vs[1], rs[1] * ws[1], Es[1]};
 #pragma unroll
-      for (int k = 0; k < 5; k++) Fr[k] = Fs[1][k] + SR * (Ust[k] - Us[1][k]);
+      for (int k = 0; k < 5; k++) Fr[k] = madd(SR, Ust[k] - Us[1][k], Fs[1][k]);
     } else {
       const T sg = bx > T(0) ? T(1) : bx < T(0) ? T(-1) : T(0);
-      const T isum = T(1) / (sr[0] + sr[1]);
-      const T vss = ((sr[0] * vs[0] + sr[1] * vs[1]) + (bys[1] - bys[0]) * sg) * isum;
-      const T wss = ((sr[0] * ws[0] + sr[1] * ws[1]) + (bzs[1] - bzs[0]) * sg) * isum;
-      const T byss = ((sr[0] * bys[1] + sr[1] * bys[0]) + sr[0] * sr[1] * (vs[1] - vs[0]) * sg) * isum;
-      const T bzss = ((sr[0] * bzs[1] + sr[1] * bzs[0]) + sr[0] * sr[1] * (ws[1] - ws[0]) * sg) * isum;
-      const T vBss = SM * bx + vss * byss + wss * bzss;
+      const T isum = rcp_k(sr[0] + sr[1]);
+      const T vss = madd(bys[1] - bys[0], sg, madd(sr[1], vs[1], sr[0] * vs[0])) * isum;
+      const T wss = madd(bzs[1] - bzs[0], sg, madd(sr[1], ws[1], sr[0] * ws[0])) * isum;
+      const T byss = madd(sr[0] * sr[1] * (vs[1] - vs[0]), sg, madd(sr[1], bys[0], sr[0] * bys[1])) * isum;
+      const T bzss = madd(sr[0] * sr[1] * (ws[1] - ws[0]), sg, madd(sr[1], bzs[0], sr[0] * bzs[1])) * isum;
+      const T vBss = madd(wss, bzss, madd(vss, byss, SM * bx));
       // the side of the contact that holds x/t = 0 (selects, no indexing by
       // a run-time side)
       const bool left = SM >= T(0);
       const T rsa = left ? rs[0] : rs[1], vsa = left ? vs[0] : vs[1], wsa = left ? ws[0] : ws[1];
       const T bysa = left ? bys[0] : bys[1], bzsa = left ? bzs[0] : bzs[1];
-      const T vBsa = SM * bx + vsa * bysa + wsa * bzsa;
-      const T Ess = left ? Es[0] - sr[0] * (vBsa - vBss) * sg : Es[1] + sr[1] * (vBsa - vBss) * sg;
+      const T vBsa = madd(wsa, bzsa, madd(vsa, bysa, SM * bx));
+      const T Ess = left ? nmadd(sr[0] * (vBsa - vBss), sg, Es[0]) : madd(sr[1] * (vBsa - vBss), sg, Es[1]);
       const T Ust[5] = {rsa, rsa * SM, rsa * vsa, rsa * wsa, left ? Es[0] : Es[1]};
       const T Uss[5] = {rsa, rsa * SM, rsa * vss, rsa * wss, Ess};
       const T Sst = left ? SsL : SsR, Saa = left ? SL : SR;
 #pragma unroll
       for (int k = 0; k < 5; k++) {
         const T Fa = left ? Fs[0][k] : Fs[1][k], Ua = left ? Us[0][k] : Us[1][k];
-        Fr[k] = ((Fa + Sst * Uss[k]) - (Sst - Saa) * Ust[k]) - Saa * Ua;
+        Fr[k] = nmadd(Saa, Ua, nmadd(Sst - Saa, Ust[k], madd(Sst, Uss[k], Fa)));
       }
     }
   }

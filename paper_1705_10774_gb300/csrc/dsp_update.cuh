@@ -131,6 +131,7 @@ struct TileShared {
   int n[3][TABMAX];
   double red[NT / 32];
   int fallback;
+  int least;   // FP32 lower bound (bits) on the tile's largest new signal speed
   int floors;  // new cells whose pressure recovery took the floor
 };
 
@@ -144,6 +145,70 @@ __device__ __forceinline__ int axis_value(AxisC<V>) { return V; }
 
 __device__ __forceinline__ int floordiv(int a, int b) { return a >= 0 ? a / b : -((-a + b - 1) / b); }
 __device__ __forceinline__ int posmod(int a, int b) { const int r = a % b; return r < 0 ? r + b : r; }
+
+// Owner table of a padded tile (patch P of level lev at time tP): every block
+// of the level's map from (bx0, by0, bz0) on, nbx x nby x nbz of them, with
+// the slices of its owning patch that supply time tP (pick_slices: a slice
+// at exactly tP is copied, else two or three are inter- or extrapolated in
+// time).  A block whose values come from the other level points at the
+// patch's cross-level guard buffer, filled for time tP just before this
+// update.  Returns whether this thread's entries need a blend.
+template <typename T, int NT, bool CONC>
+__device__ __forceinline__ int owner_table(const DevCtx &c, int P, int lev, double tP, int bx0, int by0, int bz0,
+                                           int nbx, int nby, int nbz, TileShared<T, NT> &S) {
+  const PatchGeo &gp = c.geo[P];
+  const int *const gmap = c.gmap[lev];
+  const int *const bsz = c.bsz[lev];
+  const int *const mapd = c.mapd[lev];
+  const T **srcA = S.srcA;
+  int my_blend = 0;
+  for (int e = threadIdx.x; e < nbx * nby * nbz; e += NT) {
+    const int bx = bx0 + e % nbx, by = by0 + (e / nbx) % nby, bz = bz0 + e / (nbx * nby);
+    const int wx = posmod(bx, mapd[0]), wy = posmod(by, mapd[1]), wz = posmod(bz, mapd[2]);
+    const int Q = gmap[((long long)wz * mapd[1] + wy) * mapd[0] + wx];
+    if (Q < 0) {
+      // the cross-level guard buffer: a patch of n+4 cells at lo-2, in P's
+      // own (unwrapped) coordinates
+      for (int d = 0; d < 3; d++) {
+        S.lo[d][e] = gp.lo[d] - 2;
+        S.n[d][e] = gp.n[d] + 4;
+      }
+      srcA[e] = (const T *)c.gbuf + c.gofs[P];
+      S.blend[e] = 0;
+      continue;
+    }
+    const PatchGeo &gq = c.geo[Q];
+    S.lo[0][e] = gq.lo[0] + (bx - wx) * bsz[0];
+    S.lo[1][e] = gq.lo[1] + (by - wy) * bsz[1];
+    S.lo[2][e] = gq.lo[2] + (bz - wz) * bsz[2];
+    S.n[0][e] = gq.n[0];
+    S.n[1][e] = gq.n[1];
+    S.n[2][e] = gq.n[2];
+    const T *base = (const T *)c.slab + gq.off;
+    SlicePick pk;
+    if (pick_slices<CONC>(c, Q, tP, pk) != DSP_OK) {
+      pk.n = 1;
+      pk.s[0] = newest<CONC>(c, Q);
+      set_error(c, DSP_ERR_BRACKET, P, -1);
+    }
+    srcA[e] = base + (long long)pk.s[0] * c.slot_stride;
+    int bl = 0;
+    if (pk.n >= 2) {
+      bl = pk.n | ((pk.s[1] - pk.s[0] + 16) << 2) | ((pk.n == 3 ? pk.s[2] - pk.s[0] + 16 : 16) << 8);
+      my_blend = 1;
+    }
+    S.blend[e] = bl;
+#pragma unroll
+    for (int q = 0; q < 3; q++) S.wgt[q][e] = q < pk.n ? (T)pk.w[q] : T(0);
+  }
+  return my_blend;
+}
+
+}  // namespace dsp
+
+#include "dsp_march.cuh"
+
+namespace dsp {
 
 // Advance one tile of patch P by dt (all threads of the block take part).
 // On return the tile's new cells, faces and signal speed are written.  CONC:
@@ -220,62 +285,14 @@ __device__ __forceinline__ void process_tile(const DevCtx &c, const int P, const
   const T *const own = (const T *)c.slab + (long long)Lp * c.slot_stride + gp.off;
   T *const dst = (T *)c.slab + (long long)((Lp + 1) % c.ns) * c.slot_stride + gp.off;
 
-  // Owner table of the padded tile: every block of the level's map that
-  // cells in [x0-2, x0+tx+2] x [y0-2, y0+ty+2] x [z0-2, z0+tz+2] fall in, with
-  // the slices of its owning patch that supply time tP (pick_slices: a slice
-  // at exactly tP is copied, else two or three are inter- or extrapolated in
-  // time).  A block whose values
-  // come from the other level points at the patch's cross-level guard
-  // buffer, filled for time tP just before this update.
-  const int *const gmap = c.gmap[lev];
   const int *const bsz = c.bsz[lev];
-  const int *const mapd = c.mapd[lev];
   const float *const binv = c.binv[lev];
   const int bx0 = floordiv(lox + x0 - 2, bsz[0]), by0 = floordiv(loy + y0 - 2, bsz[1]),
             bz0 = floordiv(loz + z0 - 2, bsz[2]);
   const int nbx = floordiv(lox + x0 + tx + 2, bsz[0]) - bx0 + 1;
   const int nby = floordiv(loy + y0 + ty + 2, bsz[1]) - by0 + 1;
   const int nbz = floordiv(loz + z0 + tz + 2, bsz[2]) - bz0 + 1;
-  int my_blend = 0;
-  for (int e = tid; e < nbx * nby * nbz; e += NT) {
-    const int bx = bx0 + e % nbx, by = by0 + (e / nbx) % nby, bz = bz0 + e / (nbx * nby);
-    const int wx = posmod(bx, mapd[0]), wy = posmod(by, mapd[1]), wz = posmod(bz, mapd[2]);
-    const int Q = gmap[((long long)wz * mapd[1] + wy) * mapd[0] + wx];
-    if (Q < 0) {
-      // the cross-level guard buffer: a patch of n+4 cells at lo-2, in P's
-      // own (unwrapped) coordinates
-      for (int d = 0; d < 3; d++) {
-        S.lo[d][e] = gp.lo[d] - 2;
-        S.n[d][e] = gp.n[d] + 4;
-      }
-      srcA[e] = (const T *)c.gbuf + c.gofs[P];
-      S.blend[e] = 0;
-      continue;
-    }
-    const PatchGeo &gq = c.geo[Q];
-    S.lo[0][e] = gq.lo[0] + (bx - wx) * bsz[0];
-    S.lo[1][e] = gq.lo[1] + (by - wy) * bsz[1];
-    S.lo[2][e] = gq.lo[2] + (bz - wz) * bsz[2];
-    S.n[0][e] = gq.n[0];
-    S.n[1][e] = gq.n[1];
-    S.n[2][e] = gq.n[2];
-    const T *base = (const T *)c.slab + gq.off;
-    SlicePick pk;
-    if (pick_slices<CONC>(c, Q, tP, pk) != DSP_OK) {
-      pk.n = 1;
-      pk.s[0] = newest<CONC>(c, Q);
-      set_error(c, DSP_ERR_BRACKET, P, -1);
-    }
-    srcA[e] = base + (long long)pk.s[0] * c.slot_stride;
-    int bl = 0;
-    if (pk.n >= 2) {
-      bl = pk.n | ((pk.s[1] - pk.s[0] + 16) << 2) | ((pk.n == 3 ? pk.s[2] - pk.s[0] + 16 : 16) << 8);
-      my_blend = 1;
-    }
-    S.blend[e] = bl;
-#pragma unroll
-    for (int q = 0; q < 3; q++) S.wgt[q][e] = q < pk.n ? (T)pk.w[q] : T(0);
-  }
+  const int my_blend = owner_table<T, NT, CONC>(c, P, lev, tP, bx0, by0, bz0, nbx, nby, nbz, S);
   if (tid == 0) {
     s_fallback = 0;
     S.floors = 0;
@@ -1154,6 +1171,18 @@ __device__ __forceinline__ void process_tile(const DevCtx &c, const int P, const
 #undef F5
 }
 
+template <typename T, int TX, int TY, int NT, bool CONC, int RS, int NI>
+__device__ __forceinline__ void update_tile(const DevCtx &c, int P, double dt, int tile, T *sm, TileShared<T, NT> &S) {
+  if constexpr (NI != 0) process_tile<T, TX, TY, NT, CONC, RS, NI>(c, P, dt, tile, sm, S);
+  else march_tile<T, TX, TY, NT, CONC, RS>(c, P, dt, tile, sm, S);
+}
+// its shared memory in bytes
+template <typename T, int TX, int TY, int NI>
+constexpr size_t update_smem() {
+  if constexpr (NI != 0) return sizeof(T) * (size_t)Lay<TX, TY, NI>::total;
+  else return sizeof(T) * (size_t)March<T, TX, TY>::total;
+}
+
 // Sweep dispatcher: every (ready patch, tile) work item of size classes
 // [cls, cls_end) in the current work list (grouped by class), grid-strided
 // over a persistent grid.
@@ -1175,8 +1204,7 @@ __global__ void __launch_bounds__(NT, MINB) update_kernel(DevCtx c, int cls, int
       else hi = mid - 1;
     }
     const int r = c.Rk[lo];
-    process_tile<T, TX, TY, NT, false, RS, NI>(c, c.R[r], c.dtR[r], w - c.work_off[lo], reinterpret_cast<T *>(smraw),
-                                               S);
+    update_tile<T, TX, TY, NT, false, RS, NI>(c, c.R[r], c.dtR[r], w - c.work_off[lo], reinterpret_cast<T *>(smraw), S);
   }
 }
 
@@ -1307,7 +1335,7 @@ __global__ void __launch_bounds__(NT, MINB) queue_kernel(DevCtx c, double t_end)
     if (s_exit) return;
     const int P = s_P, tile = s_tile;
     const double dt = s_dt;
-    process_tile<T, TX, TY, NT, true, RS, NI>(c, P, dt, tile, reinterpret_cast<T *>(smraw), S);
+    update_tile<T, TX, TY, NT, true, RS, NI>(c, P, dt, tile, reinterpret_cast<T *>(smraw), S);
     if (tid == 0) {
       __threadfence();
       const int k = atomicAdd(&c.tiles_done[P], 1);
@@ -1333,14 +1361,14 @@ template <typename T, int TX, int TY, int NT, int MINB, int VARIANT, int RS, int
 int launch_update(const DevCtx &c, int grid, void *stream, int cls, int cls_end) {
   // the shared-memory attribute was set by update_grid when the context was
   // created (a launch may be inside a stream capture)
-  const size_t smem = sizeof(T) * (size_t)Lay<TX, TY, NI>::total;
+  const size_t smem = update_smem<T, TX, TY, NI>();
   update_kernel<T, TX, TY, NT, MINB, VARIANT, RS, NI><<<grid, NT, smem, (cudaStream_t)stream>>>(c, cls, cls_end);
   return cudaGetLastError() == cudaSuccess ? DSP_OK : DSP_ERR_CUDA;
 }
 
 template <typename T, int TX, int TY, int NT, int MINB, int VARIANT, int RS, int NI>
 int launch_queue(const DevCtx &c, int grid, double t_end, void *stream) {
-  const size_t smem = sizeof(T) * (size_t)Lay<TX, TY, NI>::total;
+  const size_t smem = update_smem<T, TX, TY, NI>();
   static bool configured = false;
   if (!configured) {
     if (cudaFuncSetAttribute(queue_kernel<T, TX, TY, NT, MINB, VARIANT, RS, NI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1362,7 +1390,7 @@ int launch_queue(const DevCtx &c, int grid, double t_end, void *stream) {
 
 template <typename T, int TX, int TY, int NT, int MINB, int VARIANT, int RS, int NI>
 int update_grid(const DevCtx &c, int cls, int cls_end) {
-  const size_t smem = sizeof(T) * (size_t)Lay<TX, TY, NI>::total;
+  const size_t smem = update_smem<T, TX, TY, NI>();
   cudaFuncSetAttribute(update_kernel<T, TX, TY, NT, MINB, VARIANT, RS, NI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   int dev = 0, nsm = 0, per = 0;
   cudaGetDevice(&dev);

@@ -13,18 +13,18 @@
 #pragma once
 
 #define DSP_VARIANT_LIST_ALL(X)        \
-  X(0, double, 16, 8, 256, 1, 0, 0, 0)    \
-  X(1, double, 16, 8, 384, 1, 0, 0, 0)    \
-  X(2, double, 16, 8, 256, 1, 2, 0, 0)    \
-  X(3, double, 16, 8, 384, 1, 2, 0, 0)    \
-  X(4, double, 16, 8, 512, 1, 2, 0, 0)    \
-  X(5, float, 16, 8, 256, 2, 1, 0, 0)     \
-  X(6, float, 16, 8, 512, 1, 1, 0, 0)     \
-  X(7, float, 32, 8, 256, 1, 1, 0, 0)     \
-  X(8, float, 16, 16, 256, 1, 1, 0, 0)    \
-  X(9, double, 16, 8, 256, 1, 0, 1, 0)    \
-  X(10, double, 16, 8, 256, 1, 2, 1, 0)   \
-  X(11, float, 16, 8, 256, 2, 1, 1, 0)  \
+  X(0, double, 16, 8, 192, 1, 0, 0, 0)    \
+  X(1, double, 8, 8, 128, 2, 0, 0, 0)    \
+  X(2, double, 16, 8, 192, 1, 2, 0, 0)    \
+  X(3, double, 8, 8, 128, 2, 2, 0, 0)    \
+  X(4, double, 16, 12, 256, 1, 2, 0, 0)    \
+  X(5, float, 16, 8, 192, 2, 1, 0, 0)     \
+  X(6, float, 16, 8, 192, 1, 1, 0, 0)     \
+  X(7, float, 32, 8, 384, 1, 1, 0, 0)     \
+  X(8, float, 16, 16, 352, 1, 1, 0, 0)    \
+  X(9, double, 16, 8, 192, 1, 0, 1, 0)    \
+  X(10, double, 16, 8, 192, 1, 2, 1, 0)   \
+  X(11, float, 16, 8, 192, 2, 1, 1, 0)  \
   X(12, double, 16, 4, 128, 1, 0, 0, 1) \
   X(13, double, 16, 4, 128, 1, 2, 0, 1) \
   X(14, float, 16, 8, 256, 1, 1, 0, 1) \
@@ -34,12 +34,12 @@
   X(18, double, 16, 4, 256, 1, 0, 1, 1) \
   X(19, double, 16, 4, 256, 1, 2, 1, 1) \
   X(20, float, 16, 8, 256, 1, 1, 1, 1)   \
-  X(21, float, 24, 8, 256, 1, 1, 0, 0)
+  X(21, float, 24, 8, 288, 1, 1, 0, 0)
 
 #define DSP_VARIANT_LIST_CHECKED(X)    \
-  X(0, double, 16, 8, 256, 1, 0, 0, 0)    \
-  X(2, double, 16, 8, 256, 1, 2, 0, 0)    \
-  X(5, float, 16, 8, 256, 2, 1, 0, 0)
+  X(0, double, 16, 8, 192, 1, 0, 0, 0)    \
+  X(2, double, 16, 8, 192, 1, 2, 0, 0)    \
+  X(5, float, 16, 8, 192, 2, 1, 0, 0)
 
 #ifdef DSP_BOUNDS_CHECK
 #define DSP_VARIANT_LIST(X) DSP_VARIANT_LIST_CHECKED(X)

@@ -1,0 +1,65 @@
+"""The update kernel at the edges of its tile shapes: patches one cell short
+of, equal to and one cell past the tiles' extents, thin ones, and several
+tiles with a ragged last one, for every tile shape of every precision.
+
+FP64 without FMA: state, times and signal speeds equal the oracle's bit for
+bit.  The other precisions: every tile shape and z run gives the same bits,
+within 1e-11 (FP64 with FMA, the tolerance of the parity tests) or 1e-5 (FP32:
+some ten roundings of 6e-8 on each of a few dozen terms per step, two steps)
+of the oracle's largest value."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from paper_1705_10774_gb300 import build as B
+from paper_1705_10774_gb300 import ics
+from paper_1705_10774_gb300.dispatch import Dispatch
+from oracle import Oracle
+
+SIZES = [(4, 4, 4), (7, 8, 5), (16, 11, 4), (17, 9, 6), (15, 12, 7), (33, 13, 5), (31, 17, 4), (24, 8, 9), (49, 4, 4)]
+
+
+def _case(n, seed):
+    lay = ics.cartesian((2, 2, 2), n)
+    X, Y, Z = lay.base_cells
+    rng = np.random.default_rng(seed)
+    shape = (Z, Y, X)
+    A = [0.02 * lay.dx * rng.standard_normal(shape) for _ in range(3)]
+    bx, by, bz = ics.curl_faces(*A, lay.dx)
+    f = ics.Fields(rho=1 + 0.3 * rng.random(shape), v=0.5 * rng.standard_normal((3,) + shape),
+                   p=0.6 + 0.2 * rng.random(shape), bx=bx + 0.5, by=by + 0.3, bz=bz - 0.2, gamma=5.0 / 3.0)
+    return lay, ics.to_patches(lay, f)
+
+
+@pytest.mark.parametrize("precision", [0, 1, 2])
+@pytest.mark.parametrize("n", SIZES)
+def test_every_tile_shape_at_its_edges(n, precision):
+    lay, state = _case(n, sum(n))
+    kw = dict(gamma=5.0 / 3.0, cfl=0.4, base_cells=lay.base_cells, box_len=lay.box_len, time_mode=0)
+    o = Oracle(lay.n, lay.lo, **kw)
+    o.set_state(*state)
+    o.advance(max_sweeps=2)
+    ref, (_, _, speed) = o.get_state(), o.get_times()
+    scale = max(float(np.max(np.abs(a))) for a in ref)
+    first = None
+    ids = [v[0] for v in B.variants() if v[6] == precision and v[7] == 0 and v[8] == 0]
+    for vid, tile_z in [(v, 0) for v in ids] + [(-1, 0), (ids[0], 1), (ids[-1], 3)]:
+        g = Dispatch(lay.n, lay.lo, precision=precision, variant=vid, tile_z=tile_z, **kw)
+        g.set_state(*state)
+        g.advance(max_sweeps=2)
+        out = g.get_state()
+        smax = g.pack(np.arange(lay.npatch), device=False)[1][:, 2].copy()
+        g.close()
+        if first is None:
+            first = out, smax
+        for a, b in zip(out, first[0]):
+            assert np.array_equal(a, b), (vid, tile_z)
+        assert np.array_equal(smax, first[1])
+    if precision == 0:
+        assert all(np.array_equal(a, b) for a, b in zip(first[0], ref)) and np.array_equal(first[1], speed)
+    else:
+        tol = 1e-11 if precision == 2 else 1e-5
+        assert max(float(np.max(np.abs(a - b))) for a, b in zip(first[0], ref)) <= tol * scale
+        assert np.max(np.abs(first[1] - speed)) <= tol * np.max(speed)
