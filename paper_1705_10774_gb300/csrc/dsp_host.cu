@@ -26,6 +26,7 @@
 
 #include "dsp_diag.cuh"
 #include "dsp_dispatch.cuh"
+#include "dsp_fast.cuh"
 #include "dsp_internal.h"
 #include "dsp_levels.cuh"
 #include "dsp_physics.cuh"
@@ -276,13 +277,71 @@ __global__ void __launch_bounds__(PLAN_NT) plan_compact_kernel(DevCtx c, int glo
     }
   }
   if (tid == 0) c.ctl[CTL_CLS + c.ncls] = s_kb;
+  // Planes per work item.  A sweep whose tiles leave blocks idle (a few
+  // patches, or one large one) cuts each z run into m equal parts: a part of
+  // s planes costs s + 2 (its halo planes), and the sweep takes as many
+  // rounds of blocks as the items need, so the m that minimises rounds x
+  // (s + 5/2) is taken (half a plane for an item's start).  Eight patches of
+  // 16^3 (16 tiles), FP64 without FMA: 1.43 ms a sweep uncut, 0.32 ms cut; ten
+  // of 30 x 4 x 4 (20 tiles): 0.43 and 0.21 ms.  Sweeps that fill the GPU
+  // four times over are left whole.
+  {
+    constexpr int NM = 8;
+    const int cut[NM] = {1, 2, 3, 4, 6, 8, 16, 32};
+    __shared__ int s_items[NM];
+    for (int k = 0; k < c.ncls; k++) {
+      const int r0 = c.ctl[CTL_CLS + k], r1 = k + 1 < c.ncls ? c.ctl[CTL_CLS + k + 1] : s_kb;
+      const int slots = c.cls_slots[k], tz = c.cls_tz[k];
+      __syncthreads();
+      if (tid < NM) s_items[tid] = 0;
+      __syncthreads();
+      if (slots > 0 && r1 - r0 < 4 * slots) {
+        int n[NM] = {};
+        for (int r = r0 + tid; r < r1; r += PLAN_NT) {
+          const PatchGeo &g = c.geo[c.R[c.Rk[r]]];
+#pragma unroll
+          for (int m = 0; m < NM; m++) {
+            const int s = (tz + cut[m] - 1) / cut[m];
+            n[m] += g.tiles * ((g.tz + s - 1) / s);
+          }
+        }
+#pragma unroll
+        for (int m = 0; m < NM; m++) {
+          const int v = __reduce_add_sync(0xffffffffu, n[m]);
+          if (lane == 0 && v) atomicAdd(&s_items[m], v);
+        }
+      }
+      __syncthreads();
+      if (tid == 0) {
+        int best = tz;
+        if (s_items[0] > 0 && s_items[0] < 4 * slots) {
+          float cost = 3e38f;
+          for (int m = 0; m < NM; m++) {
+            const int s = (tz + cut[m] - 1) / cut[m];
+            const float v = (float)((s_items[m] + slots - 1) / slots) * ((float)s + 2.5f);
+            if (v < cost) {
+              cost = v;
+              best = s;
+            }
+          }
+        }
+        c.ctl[CTL_ZRUN + k] = best;
+      }
+    }
+    __syncthreads();
+  }
   // work offsets: work-list entry i owns update work items [work_off[i], work_off[i+1])
   __shared__ int s_woff;
   if (tid == 0) s_woff = 0;
   __syncthreads();
   for (int chunk = 0; chunk < nr; chunk += PLAN_NT) {
     const int r = chunk + tid;
-    const int v = r < nr ? c.geo[c.R[c.Rk[r]]].tiles : 0;
+    int v = 0;
+    if (r < nr) {
+      const PatchGeo &g = c.geo[c.R[c.Rk[r]]];
+      const int s = c.ctl[CTL_ZRUN + g.cls];
+      v = g.tiles * ((g.tz + s - 1) / s);
+    }
     int incl = v;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -325,46 +384,105 @@ __global__ void __launch_bounds__(PLAN_NT) plan_compact_kernel(DevCtx c, int glo
   }
 }
 
-// Signal speed and positivity of slice s of every patch (one block per patch).
+// Blocks that share one patch in the kernels that pass over whole patches: a
+// piece of at least 4096 values (or cells), and no more blocks in all than
+// fill the GPU a few times, so that one large patch is spread over every SM
+// (one 128^3 patch in FP64, loaded, advanced two sweeps and read: 149 ms with
+// one block per patch, 110 ms of it loading and reading; now 0.26 ms of 20).
+int patch_parts(long long values, int patches) {
+  const long long most = std::max<long long>(1, 2432 / std::max(1, patches));
+  return (int)std::max<long long>(1, std::min<long long>(most, values / 4096));
+}
+
+// Signal speed and positivity of slice `slot` of patches [first, first +
+// count): blockIdx.y of gridDim.y blocks takes every gridDim.y-th run of
+// blockDim.x cells of patch first + blockIdx.x; the slice's speed was zeroed.
+// FP64 (without non-ideal terms): a cell's speed is bounded in FP32 and
+// evaluated in FP64 only if it may exceed the largest lower bound seen (the
+// maximum is the same value; in FP64 throughout the pass took 31 ms for
+// 134M cells, FP64-pipe bound).
 template <typename T>
-__global__ void smax_kernel(DevCtx c, int slot, int first, int count) {
+__global__ void __launch_bounds__(256) smax_kernel(DevCtx c, int slot, int first) {
   const int P = first + blockIdx.x;
-  if (P >= first + count) return;
   const PatchGeo &g = c.geo[P];
   const T *base = (const T *)c.slab + (long long)slot * c.slot_stride + g.off;
   const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
   const long long nc = (long long)nx * ny * nz;
   const T *bxa = base + 5 * nc, *bya = bxa + (long long)(nx + 1) * ny * nz, *bza = bya + (long long)nx * (ny + 1) * nz;
   const T gamma = (T)c.gamma;
+  const float gamma32 = (float)c.gamma;
+  const bool bounds = sizeof(T) == 8 && !(c.eta > 0.0 || c.gad > 0.0);
+  __shared__ int s_least;
+  __shared__ double red[8];
+  if (threadIdx.x == 0) s_least = 0;
+  __syncthreads();
   double m = 0.0;
-  for (long long id = threadIdx.x; id < nc; id += blockDim.x) {
-    const int i = (int)(id % nx), j = (int)((id / nx) % ny), k = (int)(id / ((long long)nx * ny));
-    T W[8];
-    prim(base[id], base[nc + id], base[2 * nc + id], base[3 * nc + id], base[4 * nc + id],
-         bxa[((long long)k * ny + j) * (nx + 1) + i], bxa[((long long)k * ny + j) * (nx + 1) + i + 1],
-         bya[((long long)k * (ny + 1) + j) * nx + i], bya[((long long)k * (ny + 1) + j + 1) * nx + i],
-         bza[((long long)k * ny + j) * nx + i], bza[((long long)(k + 1) * ny + j) * nx + i], gamma, W);
-    if (!(W[RHO] > T(0)) || !(W[PR] > T(0))) set_status(c, DSP_ERR_UNPHYSICAL, P);
-    T sig = signal_sum(W, gamma);
-    if (c.eta > 0.0 || c.gad > 0.0)
-      sig = tmax(sig, nonideal_speed(W, c.cfl, c.eta, c.gad, c.rhoi, c.cohm, c.cad, ldexp(c.dx, -g.level)));
-    m = fmax(m, (double)sig);
+  const long long step = (long long)gridDim.y * blockDim.x;
+  for (long long id0 = (long long)blockIdx.y * blockDim.x; id0 < nc; id0 += step) {
+    const long long id = id0 + threadIdx.x;
+    const bool in = id < nc;
+    T U[5], f[6];
+    if (in) {
+      const int row = (int)(id / nx), k = row / ny;
+#pragma unroll
+      for (int q = 0; q < 5; q++) U[q] = base[q * nc + id];
+      f[0] = bxa[id + row];
+      f[1] = bxa[id + row + 1];
+      f[2] = bya[id + (long long)k * nx];
+      f[3] = bya[id + (long long)k * nx + nx];
+      f[4] = bza[id];
+      f[5] = bza[id + (long long)nx * ny];
+    }
+    bool eval = in;
+    if constexpr (sizeof(T) == 8) {
+      if (bounds) {
+        float above = 0.f, below = 0.f;
+        if (in) fast::signal_bounds(U, f[0], f[1], f[2], f[3], f[4], f[5], gamma32, above, below);
+        const int w = __reduce_max_sync(0xffffffffu, __float_as_int(fmaxf(below, 0.f)));
+        const int least = max(w, *(volatile int *)&s_least);
+        if ((threadIdx.x & 31) == 0 && w == least) atomicMax(&s_least, w);
+        eval = in && !(above < __int_as_float(least));
+      }
+    }
+    if (eval) {
+      T W[8];
+      prim(U[0], U[1], U[2], U[3], U[4], f[0], f[1], f[2], f[3], f[4], f[5], gamma, W);
+      if (!(W[RHO] > T(0)) || !(W[PR] > T(0))) set_status(c, DSP_ERR_UNPHYSICAL, P);
+      T sig = signal_sum(W, gamma);
+      if (c.eta > 0.0 || c.gad > 0.0)
+        sig = tmax(sig, nonideal_speed(W, c.cfl, c.eta, c.gad, c.rhoi, c.cohm, c.cad, ldexp(c.dx, -g.level)));
+      m = fmax(m, (double)sig);
+    }
   }
-  __shared__ double red[32];
   for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
   __syncthreads();
-  if (threadIdx.x < 32) {
-    double u = threadIdx.x < blockDim.x / 32 ? red[threadIdx.x] : 0.0;
-    for (int o = 16; o > 0; o >>= 1) u = fmax(u, __shfl_xor_sync(0xffffffffu, u, o));
-    if (threadIdx.x == 0) c.smax_slot[(long long)P * c.ns + slot] = u;
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; w++) m = fmax(m, red[w]);
+    atomicMax((unsigned long long *)&c.smax_slot[(long long)P * c.ns + slot], (unsigned long long)__double_as_longlong(m));
   }
+}
+
+// Part blockIdx.y of gridDim.y of n values, as four loads in flight a thread.
+template <typename D, typename S>
+__device__ __forceinline__ void copy_part(D *d, const S *s, long long n) {
+  const long long step = (long long)gridDim.y * blockDim.x;
+  long long l = (long long)blockIdx.y * blockDim.x + threadIdx.x;
+  for (; l + 3 * step < n; l += 4 * step) {
+    const S a = s[l], b = s[l + step], e = s[l + 2 * step], f = s[l + 3 * step];
+    d[l] = (D)a;
+    d[l + step] = (D)b;
+    d[l + 2 * step] = (D)e;
+    d[l + 3 * step] = (D)f;
+  }
+  for (; l < n; l += step) d[l] = (D)s[l];
 }
 
 // Copy between the caller's four arrays (patches [first, first+count)) and
 // the slices: dir 0 loads slot 0, dir 1 stores each patch's newest slot.
+// gridDim.y blocks share each patch.
 template <typename TS, typename TU>
-__global__ void xfer_kernel(DevCtx c, int first, int count, TU *U, TU *bx, TU *by, TU *bz, int dir) {
+__global__ void __launch_bounds__(256) xfer_kernel(DevCtx c, int first, int count, TU *U, TU *bx, TU *by, TU *bz, int dir) {
   TU *arr[4] = {U, bx, by, bz};
   for (int P = first + blockIdx.x; P < first + count; P += gridDim.x) {
     const PatchGeo &g = c.geo[P];
@@ -373,14 +491,11 @@ __global__ void xfer_kernel(DevCtx c, int first, int count, TU *U, TU *bx, TU *b
                               (long long)g.n[0] * (g.n[1] + 1) * g.n[2], (long long)g.n[0] * g.n[1] * (g.n[2] + 1)};
     const int s = dir == 0 ? 0 : c.latest[P];
     TS *slot = (TS *)c.slab + (long long)s * c.slot_stride + g.off;
-    long long so = 0;
     for (int f = 0; f < 4; f++) {
       TU *a = arr[f] + (c.coff[f * (c.np + 1) + P] - c.coff[f * (c.np + 1) + first]);
-      for (long long l = threadIdx.x; l < per[f]; l += blockDim.x) {
-        if (dir == 0) slot[so + l] = (TS)a[l];
-        else a[l] = (TU)slot[so + l];
-      }
-      so += per[f];
+      if (dir == 0) copy_part(slot, a, per[f]);
+      else copy_part(a, slot, per[f]);
+      slot += per[f];
     }
   }
 }
@@ -390,43 +505,40 @@ __global__ void xfer_kernel(DevCtx c, int first, int count, TU *U, TU *bx, TU *b
 // its time parameters.  dir 0 (pack): newest slice -> buf + off[k], meta[k] =
 // (time, last step, signal speed).  dir 1 (unpack): buf + off[k] -> the slot
 // after the newest, which then becomes the newest with meta's time, step and
-// signal speed.  One block per listed patch (the patches are distinct).
+// signal speed.  gridDim.y blocks share each listed patch (the patches are
+// distinct); package_meta_kernel moves the times afterwards, once every block
+// has read which slot is the newest.
 template <typename T>
-__global__ void package_kernel(DevCtx c, const int *ids, const long long *off, int count, T *buf, double *meta,
-                               int dir) {
-  const int k = blockIdx.x;
-  if (k >= count) return;
-  const int P = ids[k];
-  const PatchGeo &g = c.geo[P];
-  const long long nc = (long long)g.n[0] * g.n[1] * g.n[2];
-  const long long len = 5 * nc + (long long)(g.n[0] + 1) * g.n[1] * g.n[2] + (long long)g.n[0] * (g.n[1] + 1) * g.n[2] +
-                        (long long)g.n[0] * g.n[1] * (g.n[2] + 1);
+__global__ void __launch_bounds__(256) package_kernel(DevCtx c, const int *ids, const long long *off, T *buf, int dir) {
+  const int k = blockIdx.x, P = ids[k];
   const int L = c.latest[P];
   const int s = dir == 0 ? L : (L + 1) % c.ns;
-  T *slot = (T *)c.slab + (long long)s * c.slot_stride + g.off;
+  T *slot = (T *)c.slab + (long long)s * c.slot_stride + c.geo[P].off;
   T *pkg = buf + off[k];
-  for (long long l = threadIdx.x; l < len; l += blockDim.x) {
-    if (dir == 0) pkg[l] = slot[l];
-    else slot[l] = pkg[l];
-  }
-  if (threadIdx.x == 0) {
-    const long long ts = (long long)P * c.ns;
-    if (dir == 0) {
-      meta[3 * k] = c.t_slot[ts + L];
-      meta[3 * k + 1] = c.dt_last[P];
-      meta[3 * k + 2] = c.smax_slot[ts + L];
-    } else {
-      c.t_slot[ts + s] = meta[3 * k];
-      c.dt_last[P] = meta[3 * k + 1];
-      c.smax_slot[ts + s] = meta[3 * k + 2];
-      c.latest[P] = s;
-    }
+  if (dir == 0) copy_part(pkg, slot, off[k + 1] - off[k]);
+  else copy_part(slot, pkg, off[k + 1] - off[k]);
+}
+__global__ void __launch_bounds__(256) package_meta_kernel(DevCtx c, const int *ids, int count, double *meta, int dir) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= count) return;
+  const int P = ids[k], L = c.latest[P], s = (L + 1) % c.ns;
+  const long long ts = (long long)P * c.ns;
+  if (dir == 0) {
+    meta[3 * k] = c.t_slot[ts + L];
+    meta[3 * k + 1] = c.dt_last[P];
+    meta[3 * k + 2] = c.smax_slot[ts + L];
+  } else {
+    c.t_slot[ts + s] = meta[3 * k];
+    c.dt_last[P] = meta[3 * k + 1];
+    c.smax_slot[ts + s] = meta[3 * k + 2];
+    c.latest[P] = s;
   }
 }
 
 __global__ void reset_times_kernel(DevCtx c, int first, int count, double t0) {
   for (int P = first + blockIdx.x * blockDim.x + threadIdx.x; P < first + count; P += gridDim.x * blockDim.x) {
     for (int s = 0; s < c.ns; s++) c.t_slot[(long long)P * c.ns + s] = s == 0 ? t0 : __longlong_as_double(0x7ff8000000000000ll);
+    c.smax_slot[(long long)P * c.ns] = 0.0;  // the loaded slice's speed is an atomic maximum
     c.latest[P] = 0;
     c.dt_last[P] = 0.0;
   }
@@ -476,13 +588,14 @@ __global__ void queue_init_kernel(DevCtx c, double t_end) {
   }
 }
 
-// Per-patch diagnostics of the newest slice (dsp_diag.cuh): one block per
-// patch, with the patch's own level's cell volume.
+// Diagnostics of the newest slice (dsp_diag.cuh): gridDim.y blocks share each
+// patch, with the patch's own level's cell volume; a record per block.
 template <typename T>
 __global__ void __launch_bounds__(DIAG_NT) diag_kernel(DevCtx c, double *out) {
   const int P = blockIdx.x;
+  out += ((long long)P * gridDim.y + blockIdx.y) * DIAG_PER;
   if (c.owned && !c.owned[P]) {  // a virtual patch: its owner counts it
-    if (threadIdx.x < DIAG_PER) out[(long long)P * DIAG_PER + threadIdx.x] = 0.0;
+    if (threadIdx.x < DIAG_PER) out[threadIdx.x] = 0.0;
     return;
   }
   const PatchGeo &g = c.geo[P];
@@ -491,7 +604,7 @@ __global__ void __launch_bounds__(DIAG_NT) diag_kernel(DevCtx c, double *out) {
   const long long nc = (long long)nx * ny * nz;
   const T *bxa = base + 5 * nc, *bya = bxa + (long long)(nx + 1) * ny * nz, *bza = bya + (long long)nx * (ny + 1) * nz;
   const double dxl = ldexp(c.dx, -g.level);
-  diag_patch<T>(base, bxa, bya, bza, nx, ny, nz, dxl * dxl * dxl, out + (long long)P * DIAG_PER);
+  diag_patch<T>(base, bxa, bya, bza, nx, ny, nz, dxl * dxl * dxl, out, blockIdx.y, gridDim.y);
 }
 
 int launch_queue(dsp_ctx *c, double t_end) { return c->var->launch_queue(c->d, c->grid_update, t_end, c->stream); }
@@ -522,6 +635,10 @@ void make_groups(dsp_ctx *c) {
       c->grp_hi[c->ngrp] = k + 1;
       c->ngrp++;
     }
+  }
+  for (int k = 0; k < MAXCLS; k++) {
+    c->d.cls_slots[k] = c->prm.dispatcher == 1 && k < c->ncls ? c->var_cls[k]->slots() : 0;
+    c->d.cls_tz[k] = c->tz_cls[k];
   }
   for (int k = 0; k < c->ncls; k++) c->grid_cls[k] = c->var_cls[k]->grid(c->d, k, k + 1);
   for (int g = 0; g < c->ngrp; g++) c->grid_grp[g] = c->var_cls[c->grp_lo[g]]->grid(c->d, c->grp_lo[g], c->grp_hi[g]);
@@ -661,7 +778,10 @@ int ensure_staging(dsp_ctx *c, size_t bytes) {
 
 template <typename TS>
 int run_xfer(dsp_ctx *c, int first, int count, void *U, void *bx, void *by, void *bz, int dtype, int dir) {
-  const int grid = std::min(count, 4096);
+  const int np1 = c->d.np + 1;
+  long long values = 0;
+  for (int f = 0; f < 4; f++) values += c->coff[(size_t)(f * np1 + first + count)] - c->coff[(size_t)(f * np1 + first)];
+  const dim3 grid(std::min(count, 4096), patch_parts(values / count, std::min(count, 4096)));
   if (dtype == 0)
     xfer_kernel<TS, double><<<grid, 256, 0, c->stream>>>(c->d, first, count, (double *)U, (double *)bx, (double *)by,
                                                        (double *)bz, dir);
@@ -1250,8 +1370,10 @@ extern "C" int dsp_set_state(dsp_ctx *c, int32_t first, int32_t count, const voi
   CK(cudaGetLastError());
   CK(cudaMemsetAsync(c->ctl, 0, sizeof(int) * CTL_COUNT, c->stream));
   CK(cudaMemsetAsync(c->cnt, 0, sizeof(long long) * CNT_COUNT, c->stream));
-  if (c->precision != 1) smax_kernel<double><<<count, 256, 0, c->stream>>>(c->d, 0, first, count);
-  else smax_kernel<float><<<count, 256, 0, c->stream>>>(c->d, 0, first, count);
+  const long long cells = (c->coff[(size_t)(first + count)] - c->coff[(size_t)first]) / 5;
+  const dim3 grid(count, patch_parts(cells / count, count));
+  if (c->precision != 1) smax_kernel<double><<<grid, 256, 0, c->stream>>>(c->d, 0, first);
+  else smax_kernel<float><<<grid, 256, 0, c->stream>>>(c->d, 0, first);
   CK(cudaGetLastError());
   rc = read_status(c);
   if (rc) return rc;
@@ -1500,18 +1622,20 @@ extern "C" int dsp_get_schedule(dsp_ctx *c, dsp_sched_entry *buf, int64_t cap, i
 extern "C" int dsp_diagnostics(dsp_ctx *c, dsp_diag *out) {
   if (!c || !out) return DSP_ERR_INVALID_ARG;
   const int np = c->d.np;
+  const int parts = diag_parts(c->coff[(size_t)np] / 5 / np, np, INT64_MAX);
+  const int recs = np * parts;
   double *dd = nullptr;
-  CK(cudaMalloc(&dd, sizeof(double) * DIAG_PER * np));
-  if (c->precision != 1) diag_kernel<double><<<np, DIAG_NT, 0, c->stream>>>(c->d, dd);
-  else diag_kernel<float><<<np, DIAG_NT, 0, c->stream>>>(c->d, dd);
+  CK(cudaMalloc(&dd, sizeof(double) * DIAG_PER * recs));
+  if (c->precision != 1) diag_kernel<double><<<dim3(np, parts), DIAG_NT, 0, c->stream>>>(c->d, dd);
+  else diag_kernel<float><<<dim3(np, parts), DIAG_NT, 0, c->stream>>>(c->d, dd);
   cudaError_t e = cudaGetLastError();
-  std::vector<double> h((size_t)DIAG_PER * np);
+  std::vector<double> h((size_t)DIAG_PER * recs);
   if (e == cudaSuccess) e = cudaMemcpyAsync(h.data(), dd, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, c->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   cudaFree(dd);
   if (e != cudaSuccess) return fail(c, DSP_ERR_CUDA, "diagnostics: %s", cudaGetErrorString(e));
   double r[DIAG_PER];
-  diag_combine(h.data(), np, r);
+  diag_combine(h.data(), recs, r);
   out->mass = r[0];
   for (int d = 0; d < 3; d++) out->mom[d] = r[1 + d];
   out->energy = r[4];
@@ -1741,10 +1865,10 @@ int run_package(dsp_ctx *c, const int32_t *ids, int32_t count, void *buf, double
     CK(cudaMemcpyAsync(dbuf, buf, bytes, cudaMemcpyHostToDevice, c->stream));
     CK(cudaMemcpyAsync(dmeta, meta, sizeof(double) * 3 * count, cudaMemcpyHostToDevice, c->stream));
   }
-  if (c->precision == 1)
-    package_kernel<float><<<count, 256, 0, c->stream>>>(c->d, c->pk_ids, c->pk_off, count, (float *)dbuf, dmeta, dir);
-  else
-    package_kernel<double><<<count, 256, 0, c->stream>>>(c->d, c->pk_ids, c->pk_off, count, (double *)dbuf, dmeta, dir);
+  const dim3 grid(count, patch_parts(off[(size_t)count] / count, count));
+  if (c->precision == 1) package_kernel<float><<<grid, 256, 0, c->stream>>>(c->d, c->pk_ids, c->pk_off, (float *)dbuf, dir);
+  else package_kernel<double><<<grid, 256, 0, c->stream>>>(c->d, c->pk_ids, c->pk_off, (double *)dbuf, dir);
+  package_meta_kernel<<<(count + 255) / 256, 256, 0, c->stream>>>(c->d, c->pk_ids, count, dmeta, dir);
   CK(cudaGetLastError());
   if (!on_device && dir == 0) {
     CK(cudaMemcpyAsync(buf, dbuf, bytes, cudaMemcpyDeviceToHost, c->stream));

@@ -16,7 +16,8 @@ enum Ctl : int {
   CTL_ERRC = 4,     // cell (linear, patch-local) of the first error
   CTL_NOTDONE = 5,  // set by the readiness pass when some patch is behind t_end
   CTL_CLS = 8,      // [MAXCLS + 1]: first ready-list entry of each size class, then the end
-  CTL_COUNT = 16
+  CTL_ZRUN = 16,    // [MAXCLS] planes per work item of each size class in this sweep
+  CTL_COUNT = 24
 };
 
 // Patch-size classes: each distinct patch size (up to MAXCLS of them) has its
@@ -59,6 +60,8 @@ struct DevCtx {
   int ncls;                // size classes (1..MAXCLS)
   long long total_tiles;   // tiles of all patches
   long long cls_tiles[MAXCLS];  // tiles of each class's patches
+  int cls_slots[MAXCLS];   // blocks of each class's update kernel that run at once (0: z runs are not cut)
+  int cls_tz[MAXCLS];      // largest z run of each class's patches
   long long slot_stride;   // elements of one slice of all patches
   const PatchGeo *geo;     // [np]
   // per level l: the periodic box of L[l] cells per axis cut into blocks of
@@ -133,6 +136,7 @@ struct KernelVariant {
   int (*launch_update)(const DevCtx &c, int grid, void *stream, int cls, int cls_end);
   int (*launch_queue)(const DevCtx &c, int grid, double t_end, void *stream);
   int (*grid)(const DevCtx &c, int cls, int cls_end);
+  int (*slots)();  // blocks of the update kernel that run at once on the current device
 };
 
 #define DSP_DECLARE_VARIANT(id, T, TX, TY, NT, MB, PREC, RS, NI) const KernelVariant *variant_##id();

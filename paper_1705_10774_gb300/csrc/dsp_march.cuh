@@ -82,8 +82,8 @@ struct March {
 };
 
 template <typename T, int TX, int TY, int NT, bool CONC, int RS>
-__device__ __forceinline__ void march_tile(const DevCtx &c, const int P, const double dt, const int tile, T *sm,
-                                           TileShared<T, NT> &S) {
+__device__ __forceinline__ void march_tile(const DevCtx &c, const int P, const double dt, const int tile,
+                                           const int zlo, const int zrun, T *sm, TileShared<T, NT> &S) {
   using M = March<T, TX, TY>;
   static_assert(M::NTILE % 32 == 0, "whole warps of tile columns");
   static_assert(NT >= M::NEED && NT - M::NTILE >= M::NRING, "a thread per column");
@@ -107,8 +107,10 @@ __device__ __forceinline__ void march_tile(const DevCtx &c, const int P, const d
   keep(hdt);
   keep(dtdx);
   const int tix = tile % gp.nt[0], tiy = (tile / gp.nt[0]) % gp.nt[1], tiz = tile / (gp.nt[0] * gp.nt[1]);
-  const int x0 = tix * TX, y0 = tiy * TY, z0 = tiz * gp.tz;
-  const int tx = min(TX, nx - x0), ty = min(TY, ny - y0), tz = min(gp.tz, nz - z0);
+  const int x0 = tix * TX, y0 = tiy * TY, z0 = tiz * gp.tz + zlo;
+  const int zend = min(tiz * gp.tz + gp.tz, nz);  // of the whole z run
+  const int tx = min(TX, nx - x0), ty = min(TY, ny - y0), tz = min(zrun, zend - z0);
+  if (tz <= 0) return;
   const int Lp = newest<CONC>(c, P);
   const double tP = slot_time<CONC>(c, (long long)P * c.ns + Lp);
   const T *const own = (const T *)c.slab + (long long)Lp * c.slot_stride + gp.off;
@@ -395,7 +397,15 @@ __device__ __forceinline__ void march_tile(const DevCtx &c, const int P, const d
         // every face state positive: the state less its largest half slope is
         const T dr = fmax_mag(fmax_mag(dX[RHO], dY[RHO]), dZ[RHO]), dp = fmax_mag(fmax_mag(dX[PR], dY[PR]), dZ[PR]);
         if (!tpos(dn(ws[RHO], dr)) || !tpos(dn(ws[PR], dp))) {
-          atomicAdd(&S.fallback, 1);
+          // counted as 16 x 8 tiles and whole z runs meet the cell (the halo
+          // cells of each with it), whatever the tile and its part
+          const bool zc = (p >= z0 || zlo == 0) && (p < z0 + tz || z0 + tz == zend);
+          const int cx = min(max(x, 0), nx - 1), cy = min(max(y, 0), ny - 1);
+          if (zc && cx >= x0 && cx < x0 + tx && cy >= y0 && cy < y0 + ty) {
+            const int kx = 1 + (x > 0 && x % 16 == 0 && x < nx) + (x >= 0 && x % 16 == 15 && x < nx - 1);
+            const int ky = 1 + (y > 0 && y % 8 == 0 && y < ny) + (y >= 0 && y % 8 == 7 && y < ny - 1);
+            atomicAdd(&S.fallback, kx * ky);
+          }
 #pragma unroll
           for (int k = 0; k < 8; k++) { dX[k] = T(0); dY[k] = T(0); dZ[k] = T(0); ws[k] = w0[k]; }
         }

@@ -47,9 +47,9 @@ int scratch_address(double **out) {
   return DSP_OK;
 }
 
-// One block per patch (all patches of n[0] x n[1] x n[2] cells, cell size
-// dx): the per-patch reduction of dsp_diagnostics.  Every element of the
-// patch's slot in `part` is written, nothing is read first.
+// gridDim.y blocks per patch (all patches of n[0] x n[1] x n[2] cells, cell
+// size dx): the per-patch reduction of dsp_diagnostics.  Every element of the
+// block's slot in `part` is written, nothing is read first.
 template <typename T>
 __global__ void __launch_bounds__(DIAG_NT) noalloc_patch_kernel(const T *U, const T *bx, const T *by, const T *bz,
                                                                 int nx, int ny, int nz, double dx, double *part) {
@@ -58,13 +58,22 @@ __global__ void __launch_bounds__(DIAG_NT) noalloc_patch_kernel(const T *U, cons
   const long long nfx = (long long)(nx + 1) * ny * nz, nfy = (long long)nx * (ny + 1) * nz,
                   nfz = (long long)nx * ny * (nz + 1);
   diag_patch<T>(U + (long long)P * 5 * nc, bx + (long long)P * nfx, by + (long long)P * nfy, bz + (long long)P * nfz,
-                nx, ny, nz, dx * dx * dx, part + (long long)P * kPer);
+                nx, ny, nz, dx * dx * dx, part + ((long long)P * gridDim.y + blockIdx.y) * kPer, blockIdx.y, gridDim.y);
 }
 
-// One thread combines the patches in patch order into the ten values after
+// One block combines the records, in a fixed order, into the ten values after
 // the per-patch block of the scratch array.
-__global__ void noalloc_final_kernel(const double *part, int np, double *out) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) diag_combine(part, np, out);
+__global__ void __launch_bounds__(DIAG_NT) noalloc_final_kernel(const double *part, int recs, double *out) {
+  NSum acc[8];
+  for (int q = 0; q < 8; q++) acc[q].s = acc[q].c = 0.0;
+  long long mdiv = 0, mb = 0;
+  for (int r = threadIdx.x; r < recs; r += DIAG_NT) {
+#pragma unroll
+    for (int q = 0; q < 8; q++) nadd_dev(acc[q], part[(long long)r * kPer + q]);
+    mdiv = diag_max(mdiv, part[(long long)r * kPer + 8]);
+    mb = diag_max(mb, part[(long long)r * kPer + 9]);
+  }
+  diag_block(acc, mdiv, mb, out);
 }
 
 }  // namespace
@@ -79,15 +88,17 @@ extern "C" int dsp_diagnostics_noalloc(const void *U, const void *bx, const void
   int rc = scratch_address(&scratch);
   if (rc) return rc;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
+  const int parts = diag_parts((long long)n[0] * n[1] * n[2], npatch, kMax);
+  const dim3 grid(npatch, parts);
   if (dtype == 0)
-    noalloc_patch_kernel<double><<<npatch, DIAG_NT, 0, s>>>((const double *)U, (const double *)bx, (const double *)by,
+    noalloc_patch_kernel<double><<<grid, DIAG_NT, 0, s>>>((const double *)U, (const double *)bx, (const double *)by,
                                                         (const double *)bz, n[0], n[1], n[2], dx, scratch);
   else
-    noalloc_patch_kernel<float><<<npatch, DIAG_NT, 0, s>>>((const float *)U, (const float *)bx, (const float *)by,
+    noalloc_patch_kernel<float><<<grid, DIAG_NT, 0, s>>>((const float *)U, (const float *)bx, (const float *)by,
                                                        (const float *)bz, n[0], n[1], n[2], dx, scratch);
   if (cudaGetLastError() != cudaSuccess) return DSP_ERR_CUDA;
   double *result = scratch + (long long)kMax * kPer;
-  noalloc_final_kernel<<<1, 32, 0, s>>>(scratch, npatch, result);
+  noalloc_final_kernel<<<1, DIAG_NT, 0, s>>>(scratch, npatch * parts, result);
   if (cudaGetLastError() != cudaSuccess) return DSP_ERR_CUDA;
   double h[kPer];
   if (cudaMemcpyAsync(h, result, sizeof h, cudaMemcpyDeviceToHost, s) != cudaSuccess) return DSP_ERR_CUDA;

@@ -218,8 +218,8 @@ namespace dsp {
 // Poynting flux; these variants gather each plane synchronously (no copies
 // in flight) and hold three planes of faces.
 template <typename T, int TX, int TY, int NT, bool CONC, int RS, int NI>
-__device__ __forceinline__ void process_tile(const DevCtx &c, const int P, const double dt, const int tile, T *sm,
-                                             TileShared<T, NT> &S) {
+__device__ __forceinline__ void process_tile(const DevCtx &c, const int P, const double dt, const int tile,
+                                             const int zlo, const int zrun, T *sm, TileShared<T, NT> &S) {
   static_assert(TX * TY <= NT, "one updated cell per thread");
   using L = Lay<TX, TY, NI>;
   // asynchronous copies of the next plane and of the old values (sweep
@@ -278,8 +278,10 @@ __device__ __forceinline__ void process_tile(const DevCtx &c, const int P, const
   const T hdt = (T)(0.5 * dt / dxl);
   const T dtdx = (T)(dt / dxl);
   const int tix = tile % gp.nt[0], tiy = (tile / gp.nt[0]) % gp.nt[1], tiz = tile / (gp.nt[0] * gp.nt[1]);
-  const int x0 = tix * TX, y0 = tiy * TY, z0 = tiz * gp.tz;
-  const int tx = min(TX, nx - x0), ty = min(TY, ny - y0), tz = min(gp.tz, nz - z0);
+  const int x0 = tix * TX, y0 = tiy * TY, z0 = tiz * gp.tz + zlo;
+  const int zend = min(tiz * gp.tz + gp.tz, nz);  // of the whole z run
+  const int tx = min(TX, nx - x0), ty = min(TY, ny - y0), tz = min(zrun, zend - z0);
+  if (tz <= 0) return;
   const int Lp = newest<CONC>(c, P);
   const double tP = slot_time<CONC>(c, (long long)P * c.ns + Lp);
   const T *const own = (const T *)c.slab + (long long)Lp * c.slot_stride + gp.off;
@@ -694,7 +696,8 @@ __device__ __forceinline__ void process_tile(const DevCtx &c, const int P, const
           if (!tpos(rp_) || !tpos(rm_) || !tpos(pp_) || !tpos(pm_)) bad = true;
         }
         if (bad) {
-          atomicAdd(&s_fallback, 1);
+          // once for whole z runs, whatever their parts
+          if ((p >= z0 || zlo == 0) && (p < z0 + tz || z0 + tz == zend)) atomicAdd(&s_fallback, 1);
 #pragma unroll
           for (int k = 0; k < 8; k++) { dX[k] = T(0); dY[k] = T(0); dZ[k] = T(0); ws[k] = w8[k]; }
         }
@@ -1171,10 +1174,12 @@ __device__ __forceinline__ void process_tile(const DevCtx &c, const int P, const
 #undef F5
 }
 
+// Planes [zlo, zlo + zrun) of a tile's z run (cut at its end).
 template <typename T, int TX, int TY, int NT, bool CONC, int RS, int NI>
-__device__ __forceinline__ void update_tile(const DevCtx &c, int P, double dt, int tile, T *sm, TileShared<T, NT> &S) {
-  if constexpr (NI != 0) process_tile<T, TX, TY, NT, CONC, RS, NI>(c, P, dt, tile, sm, S);
-  else march_tile<T, TX, TY, NT, CONC, RS>(c, P, dt, tile, sm, S);
+__device__ __forceinline__ void update_tile(const DevCtx &c, int P, double dt, int tile, int zlo, int zrun, T *sm,
+                                            TileShared<T, NT> &S) {
+  if constexpr (NI != 0) process_tile<T, TX, TY, NT, CONC, RS, NI>(c, P, dt, tile, zlo, zrun, sm, S);
+  else march_tile<T, TX, TY, NT, CONC, RS>(c, P, dt, tile, zlo, zrun, sm, S);
 }
 // its shared memory in bytes
 template <typename T, int TX, int TY, int NI>
@@ -1203,8 +1208,11 @@ __global__ void __launch_bounds__(NT, MINB) update_kernel(DevCtx c, int cls, int
       if (c.work_off[mid] <= w) lo = mid;
       else hi = mid - 1;
     }
-    const int r = c.Rk[lo];
-    update_tile<T, TX, TY, NT, false, RS, NI>(c, c.R[r], c.dtR[r], w - c.work_off[lo], reinterpret_cast<T *>(smraw), S);
+    const int r = c.Rk[lo], P = c.R[r], item = w - c.work_off[lo];
+    // a tile's z run is cut into parts of the sweep's length
+    const int zrun = c.ctl[CTL_ZRUN + c.geo[P].cls], parts = (c.geo[P].tz + zrun - 1) / zrun;
+    update_tile<T, TX, TY, NT, false, RS, NI>(c, P, c.dtR[r], item / parts, item % parts * zrun, zrun,
+                                              reinterpret_cast<T *>(smraw), S);
   }
 }
 
@@ -1335,7 +1343,7 @@ __global__ void __launch_bounds__(NT, MINB) queue_kernel(DevCtx c, double t_end)
     if (s_exit) return;
     const int P = s_P, tile = s_tile;
     const double dt = s_dt;
-    update_tile<T, TX, TY, NT, true, RS, NI>(c, P, dt, tile, reinterpret_cast<T *>(smraw), S);
+    update_tile<T, TX, TY, NT, true, RS, NI>(c, P, dt, tile, 0, c.geo[P].tz, reinterpret_cast<T *>(smraw), S);
     if (tid == 0) {
       __threadfence();
       const int k = atomicAdd(&c.tiles_done[P], 1);
@@ -1389,17 +1397,21 @@ int launch_queue(const DevCtx &c, int grid, double t_end, void *stream) {
 }
 
 template <typename T, int TX, int TY, int NT, int MINB, int VARIANT, int RS, int NI>
-int update_grid(const DevCtx &c, int cls, int cls_end) {
+int update_slots() {
   const size_t smem = update_smem<T, TX, TY, NI>();
   cudaFuncSetAttribute(update_kernel<T, TX, TY, NT, MINB, VARIANT, RS, NI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   int dev = 0, nsm = 0, per = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, update_kernel<T, TX, TY, NT, MINB, VARIANT, RS, NI>, NT, smem);
-  if (per < 1) per = 1;
-  long long maxwork = 0;  // every patch of the classes ready
-  for (int k = cls; k < cls_end; k++) maxwork += c.cls_tiles[k];
-  long long g = (long long)nsm * per;
+  return nsm * (per < 1 ? 1 : per);
+}
+
+template <typename T, int TX, int TY, int NT, int MINB, int VARIANT, int RS, int NI>
+int update_grid(const DevCtx &c, int cls, int cls_end) {
+  long long maxwork = 0;  // every patch of the classes ready, its z runs cut to single planes
+  for (int k = cls; k < cls_end; k++) maxwork += c.cls_tiles[k] * (c.cls_slots[k] > 0 ? c.cls_tz[k] : 1);
+  const long long g = update_slots<T, TX, TY, NT, MINB, VARIANT, RS, NI>();
   return (int)(g < maxwork ? g : maxwork);
 }
 
