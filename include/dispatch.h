@@ -178,7 +178,8 @@ typedef struct {
 /* Counters of one dsp_advance call.  kernel_ms and kernel_launches are the
  * summed device time and the number of launches of the update kernel (only
  * when timing was requested); plan_launches counts the dispatcher kernels
- * (three per sweep) and, with two levels, the cross-level guard kernel.
+ * (three per sweep, one with at most 128 patches) and, with two levels, the
+ * cross-level guard kernel.
  * fallbacks counts cells whose reconstruction fell back to first order (a
  * face state with rho <= 0 or p <= 0); floors counts cells of new slices
  * whose pressure recovery took the floor p >= 1e-20 rho (both 0 on smooth

@@ -117,16 +117,17 @@ __device__ __forceinline__ int pick_slices(const DevCtx &c, int Q, double t, Sli
 // reads; the step is the power of two not above C dx / s (dx of P's level),
 // capped by dt_max,
 // halved until it divides t, and clipped to t_end.
+
+// The signal speeds of the slices of neighbour N that supply time t join M.
 template <bool CONC>
-__device__ int patch_dt(const DevCtx &c, int P, double t, double t_end, double *out) {
-  const int ns = c.ns;
-  double M = slot_smax<CONC>(c, (long long)P * ns + newest<CONC>(c, P));
-  for (int k = c.nbl_off[P]; k < c.nbl_off[P + 1]; k++) {
-    const int N = c.nbl[k];
-    SlicePick pk;
-    if (pick_slices<CONC>(c, N, t, pk) != DSP_OK) return DSP_ERR_BRACKET;
-    for (int q = 0; q < pk.n; q++) M = fmax(M, slot_smax<CONC>(c, (long long)N * ns + pk.s[q]));
-  }
+__device__ __forceinline__ int guard_speed(const DevCtx &c, int N, double t, double &M) {
+  SlicePick pk;
+  if (pick_slices<CONC>(c, N, t, pk) != DSP_OK) return DSP_ERR_BRACKET;
+  for (int q = 0; q < pk.n; q++) M = fmax(M, slot_smax<CONC>(c, (long long)N * c.ns + pk.s[q]));
+  return DSP_OK;
+}
+// The step of P at time t for the largest signal speed M.
+__device__ __forceinline__ int step_of(const DevCtx &c, int P, double t, double t_end, double M, double *out) {
   const double dtc = c.cfl * ldexp(c.dx, -c.geo[P].level) / M;
   int e;
   frexp(dtc, &e);
@@ -140,6 +141,15 @@ __device__ int patch_dt(const DevCtx &c, int P, double t, double t_end, double *
   if (dt > t_end - t) dt = t_end - t;
   *out = dt;
   return DSP_OK;
+}
+template <bool CONC>
+__device__ int patch_dt(const DevCtx &c, int P, double t, double t_end, double *out) {
+  double M = slot_smax<CONC>(c, (long long)P * c.ns + newest<CONC>(c, P));
+  for (int k = c.nbl_off[P]; k < c.nbl_off[P + 1]; k++) {
+    const int rc = guard_speed<CONC>(c, c.nbl[k], t, M);
+    if (rc != DSP_OK) return rc;
+  }
+  return step_of(c, P, t, t_end, M, out);
 }
 
 // May P overwrite its oldest slice?  Not while a neighbour that may be

@@ -130,17 +130,12 @@ constexpr int EVAL_NT = 256;
 // is t + dt, its signal speed the one the update kernel reduced, and the
 // schedule log gets (P, t, dt).  Cell counts are summed into the counters;
 // the other counters move in part 3, after every entry is written.
-__global__ void __launch_bounds__(EVAL_NT) plan_publish_kernel(DevCtx c) {
-  const int nprev = c.ctl[CTL_NREADY];
-  const long long s0 = c.cnt[CNT_NSCHED];
+__device__ void publish_part(const DevCtx &c, int r, int nprev, long long s0) {
   const int ns = c.ns;
-  __shared__ unsigned long long s_cells;
-  if (threadIdx.x == 0) s_cells = 0;
-  __syncthreads();
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
+  unsigned long long cells = 0;
   if (r < nprev) {
     const int P = c.R[r];
-    atomicAdd(&s_cells, (unsigned long long)c.geo[P].n[0] * c.geo[P].n[1] * c.geo[P].n[2]);
+    cells = (unsigned long long)c.geo[P].n[0] * c.geo[P].n[1] * c.geo[P].n[2];
     const double dt = c.dtR[r];
     const int L = c.latest[P], Ln = (L + 1) % ns;
     const double t = c.t_slot[(long long)P * ns + L];
@@ -155,31 +150,58 @@ __global__ void __launch_bounds__(EVAL_NT) plan_publish_kernel(DevCtx c) {
       c.sched[e].dt = dt;
     }
   }
-  __syncthreads();
-  if (threadIdx.x == 0 && s_cells) atomicAdd((unsigned long long *)&c.cnt[CNT_CELL_UPDATES], s_cells);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) cells += __shfl_xor_sync(0xffffffffu, cells, o);
+  if ((threadIdx.x & 31) == 0 && cells) atomicAdd((unsigned long long *)&c.cnt[CNT_CELL_UPDATES], cells);
+}
+__global__ void __launch_bounds__(EVAL_NT) plan_publish_kernel(DevCtx c) {
+  publish_part(c, blockIdx.x * blockDim.x + threadIdx.x, c.ctl[CTL_NREADY], c.cnt[CNT_NSCHED]);
 }
 
-// Part 2 (one thread per patch): Eq. (1) and the local step of
-// every ready patch; rflag/rdt per patch, and whether any patch is behind
-// t_end.
-__global__ void __launch_bounds__(EVAL_NT) plan_ready_kernel(DevCtx c, double t_end) {
-  if (c.ctl[CTL_STATUS] != 0) return;
-  const int P = blockIdx.x * blockDim.x + threadIdx.x;
-  if (P >= c.np) return;
+// Part 2 (one warp per patch, a lane per neighbour): Eq. (1) and the local
+// step of every ready patch; rflag/rdt per patch, and whether any patch is
+// behind t_end.  A thread per patch took 50 us for 4096 patches of 26
+// neighbours each (163 us with two levels), every neighbour a chain of
+// dependent loads.
+__device__ void ready_part(const DevCtx &c, int P, double t_end) {
+  const int lane = threadIdx.x & 31, ns = c.ns;
   int flag = 0;
   double dtP = 0.0;
-  const double t = c.t_slot[(long long)P * c.ns + c.latest[P]];
+  const double t = c.t_slot[(long long)P * ns + c.latest[P]];
   if (t < t_end && (!c.owned || c.owned[P])) {
-    c.ctl[CTL_NOTDONE] = 1;
-    double tr;
-    if (is_ready<false>(c, P, t_end, &tr)) {
-      const int rc = patch_dt<false>(c, P, t, t_end, &dtP);
-      if (rc != DSP_OK) set_status(c, rc, P);
-      else flag = 1;
+    if (lane == 0) c.ctl[CTL_NOTDONE] = 1;
+    const int k0 = c.nbl_off[P], k1 = c.nbl_off[P + 1];
+    bool ok = true;
+    for (int k = k0 + lane; k < k1; k += 32) {
+      const int N = c.nbl[k];
+      if (!(t <= slot_time<false>(c, (long long)N * ns + newest<false>(c, N)) + c.grace * c.dt_last[N])) ok = false;
+    }
+    ok = __all_sync(0xffffffffu, ok);
+    if (ok && c.grace > 0.0) ok = slot_free<false>(c, P);
+    if (ok) {
+      int rc = DSP_OK;
+      double M = c.smax_slot[(long long)P * ns + c.latest[P]];
+      for (int k = k0 + lane; k < k1; k += 32) rc = min(rc, guard_speed<false>(c, c.nbl[k], t, M));
+      rc = __reduce_min_sync(0xffffffffu, rc);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) M = fmax(M, __shfl_xor_sync(0xffffffffu, M, o));
+      if (rc == DSP_OK) rc = step_of(c, P, t, t_end, M, &dtP);
+      if (rc != DSP_OK) {
+        if (lane == 0) set_status(c, rc, P);
+      } else {
+        flag = 1;
+      }
     }
   }
-  c.rflag[P] = flag;
-  c.rdt[P] = dtP;
+  if (lane == 0) {
+    c.rflag[P] = flag;
+    c.rdt[P] = dtP;
+  }
+}
+__global__ void __launch_bounds__(EVAL_NT) plan_ready_kernel(DevCtx c, double t_end) {
+  if (c.ctl[CTL_STATUS] != 0) return;
+  const int P = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (P < c.np) ready_part(c, P, t_end);
 }
 
 // Block-wide exclusive scan of one flag per thread (ballot/popc per warp,
@@ -214,7 +236,21 @@ __device__ __forceinline__ int block_scan_flag(int flag, int *s_wsum, int &s_tot
 // list's entries grouped by size class, each class's kernel taking its own
 // stretch [ctl[CTL_CLS + k], ctl[CTL_CLS + k + 1]) -- with its work offsets,
 // and done / deadlock.
-__global__ void __launch_bounds__(PLAN_NT) plan_compact_kernel(DevCtx c, int global_mode, int publish_only) {
+//
+// FUSED (contexts of at most FUSE_MAX patches): parts 1 and 2 in the same
+// block and launch; with so few patches a sweep is three launches too many
+// long, not three too few wide.
+constexpr int FUSE_MAX = 128;
+template <bool FUSED>
+__global__ void __launch_bounds__(PLAN_NT) plan_compact_kernel(DevCtx c, double t_end, int global_mode, int publish_only) {
+  if constexpr (FUSED) {
+    const int nprev = c.ctl[CTL_NREADY];
+    if (threadIdx.x < FUSE_MAX) publish_part(c, threadIdx.x, nprev, c.cnt[CNT_NSCHED]);
+    __syncthreads();
+    if (!publish_only && c.ctl[CTL_STATUS] == 0)
+      for (int P = threadIdx.x >> 5; P < c.np; P += PLAN_NT / 32) ready_part(c, P, t_end);
+    __syncthreads();
+  }
   __shared__ int s_wsum[PLAN_NT / 32];
   __shared__ int s_base, s_total;
   __shared__ unsigned long long s_dtmin;
@@ -636,21 +672,38 @@ void make_groups(dsp_ctx *c) {
       c->ngrp++;
     }
   }
+  // a launch group's grid: every resident block, or one per work item if all
+  // patches were ready with their z runs cut to single planes
+  const bool cut = c->prm.dispatcher == 1;
   for (int k = 0; k < MAXCLS; k++) {
-    c->d.cls_slots[k] = c->prm.dispatcher == 1 && k < c->ncls ? c->var_cls[k]->slots() : 0;
+    c->d.cls_slots[k] = 0;
     c->d.cls_tz[k] = c->tz_cls[k];
   }
-  for (int k = 0; k < c->ncls; k++) c->grid_cls[k] = c->var_cls[k]->grid(c->d, k, k + 1);
-  for (int g = 0; g < c->ngrp; g++) c->grid_grp[g] = c->var_cls[c->grp_lo[g]]->grid(c->d, c->grp_lo[g], c->grp_hi[g]);
+  for (int g = 0; g < c->ngrp; g++) {
+    const int slots = c->var_cls[c->grp_lo[g]]->slots();
+    long long all = 0;
+    for (int k = c->grp_lo[g]; k < c->grp_hi[g]; k++) {
+      const long long items = c->d.cls_tiles[k] * (cut ? c->tz_cls[k] : 1);
+      if (cut) c->d.cls_slots[k] = slots;
+      c->grid_cls[k] = (int)std::min<long long>(slots, items);
+      all += items;
+    }
+    c->grid_grp[g] = (int)std::min<long long>(slots, all);
+  }
+  c->grid_update = c->grid_grp[0];
 }
 
 // One dispatcher step: publish the previous sweep, then (unless
 // publish_only) find the next ready list and its steps.
 int launch_plan(dsp_ctx *c, double t_end, int global_mode, int publish_only) {
   const int np = c->d.np;
+  if (np <= FUSE_MAX) {
+    plan_compact_kernel<true><<<1, PLAN_NT, 0, c->stream>>>(c->d, t_end, global_mode, publish_only);
+    return cudaGetLastError() == cudaSuccess ? DSP_OK : DSP_ERR_CUDA;
+  }
   plan_publish_kernel<<<(np + EVAL_NT - 1) / EVAL_NT, EVAL_NT, 0, c->stream>>>(c->d);
-  if (!publish_only) plan_ready_kernel<<<(np + EVAL_NT - 1) / EVAL_NT, EVAL_NT, 0, c->stream>>>(c->d, t_end);
-  plan_compact_kernel<<<1, PLAN_NT, 0, c->stream>>>(c->d, global_mode, publish_only);
+  if (!publish_only) plan_ready_kernel<<<(np + EVAL_NT / 32 - 1) / (EVAL_NT / 32), EVAL_NT, 0, c->stream>>>(c->d, t_end);
+  plan_compact_kernel<false><<<1, PLAN_NT, 0, c->stream>>>(c->d, t_end, global_mode, publish_only);
   return cudaGetLastError() == cudaSuccess ? DSP_OK : DSP_ERR_CUDA;
 }
 
@@ -683,7 +736,7 @@ double tile_cost(const KernelVariant *v) {
     case 6: return 1.40;   // FP32, 16 x 8, one block per SM
     case 7: return 1.76;   // FP32, 32 x 8
     case 8: return 1.94;   // FP32, 16 x 16
-    case 21: return 1.74;  // FP32, 24 x 8
+    case 21: return 1.90;  // FP32, 24 x 8 (slower than its share: nine warps, one block per SM)
     default: return 1.0;   // 16 x 8
   }
 }
@@ -756,7 +809,6 @@ bool install_tuning(dsp_ctx *c) {
       cudaSuccess)
     return false;
   make_groups(c);
-  c->grid_update = c->var->grid(c->d, 0, 1);
   return true;
 }
 
@@ -1352,7 +1404,6 @@ extern "C" int dsp_create(const dsp_patch_desc *patches, int32_t npatch, const d
     delete c;
     return DSP_ERR_CUDA;
   }
-  c->grid_update = var->grid(d, 0, 1);
   make_groups(c);
   *out = c;
   return DSP_OK;
@@ -1443,7 +1494,7 @@ int advance_queue(dsp_ctx *c, double t_end, const long long *c0, dsp_stats *out)
     out->status = st;
     out->kernel_ms = timing ? ms : 0.0;
     out->kernel_launches = 1;
-    out->plan_launches = 4;  // the three dispatcher kernels and the queue set-up
+    out->plan_launches = c->d.np <= FUSE_MAX ? 2 : 4;  // the dispatcher kernels and the queue set-up
     std::vector<double> t((size_t)c->d.np);
     if (dsp_get_times(c, t.data(), nullptr) == DSP_OK) {
       out->t_min = *std::min_element(t.begin(), t.end());
@@ -1525,7 +1576,8 @@ extern "C" int dsp_advance(dsp_ctx *c, double t_end, int64_t max_sweeps, dsp_sta
       if (rc) return rc;
     }
     const bool graphed = c->prm.graph && nb == batch;
-    plans += nb * (c->d.nlev > 1 ? 4 : 3);  // publish, readiness, compaction (+ cross-level guards)
+    // publish, readiness, compaction (one launch for few patches), cross-level guards
+    plans += nb * ((c->d.np <= FUSE_MAX ? 1 : 3) + (c->d.nlev > 1 ? 1 : 0));
     done_sweeps += nb;
     rc = read_status(c);
     if (rc) return rc;
@@ -1545,7 +1597,7 @@ extern "C" int dsp_advance(dsp_ctx *c, double t_end, int64_t max_sweeps, dsp_sta
     if (max_sweeps > 0 && done_sweeps >= max_sweeps) break;
   }
   if (launch_plan(c, t_end, global_mode, 1)) return fail(c, DSP_ERR_CUDA, "dispatcher kernel launch failed");
-  plans += 2;  // publish and compaction
+  plans += c->d.np <= FUSE_MAX ? 1 : 2;  // publish and compaction
   rc = read_status(c);
   if (rc) return rc;
   long long c1[CNT_COUNT];

@@ -135,7 +135,6 @@ struct KernelVariant {
   const char *name;
   int (*launch_update)(const DevCtx &c, int grid, void *stream, int cls, int cls_end);
   int (*launch_queue)(const DevCtx &c, int grid, double t_end, void *stream);
-  int (*grid)(const DevCtx &c, int cls, int cls_end);
   int (*slots)();  // blocks of the update kernel that run at once on the current device
 };
 

@@ -46,27 +46,112 @@ template <typename T>
 struct XSrc {
   const T *A, *B, *C;
   T w[3];
-  int Q, loc[3];
+  int n[3], loc[3];
 };
+
+// The other level's patches around one patch, each map block its source
+// cells lie in: the owner's slices for the patch's time, its size and the
+// periodic image of its first cell.  Built once per block of threads (one
+// entry a thread); finding owner, slices and weights again for each of a
+// thread's seven parent cells and six faces was a chain of dependent loads
+// that took most of this kernel's time.
+constexpr int XT = 256;
+template <typename T>
+struct XTab {
+  const T *A[XT];
+  long long dB[XT], dC[XT];  // element offsets of the other slices from A (0: none)
+  T w[3][XT];
+  int n[3][XT], lo[3][XT];
+  int b0[3], nb[3];
+  int ok;  // the blocks fit the table
+};
+
+// Source of patch Q for time t; 0 or an error code.
+template <typename T>
+__device__ int xl_slices(const DevCtx &c, int Q, double t, const T *&A, long long &dB, long long &dC, T w[3]) {
+  SlicePick pk;
+  if (pick_slices<false>(c, Q, t, pk) != DSP_OK) return DSP_ERR_BRACKET;
+  A = (const T *)c.slab + c.geo[Q].off + (long long)pk.s[0] * c.slot_stride;
+  dB = pk.n >= 2 ? (long long)(pk.s[1] - pk.s[0]) * c.slot_stride : 0;
+  dC = pk.n == 3 ? (long long)(pk.s[2] - pk.s[0]) * c.slot_stride : 0;
+  for (int q = 0; q < 3; q++) w[q] = q < pk.n ? (T)pk.w[q] : T(0);
+  return DSP_OK;
+}
+
+// Fill the table with the blocks of level lev from cell a to cell b (unwrapped).
+template <typename T>
+__device__ void xl_table(const DevCtx &c, int lev, const int a[3], const int b[3], double t, int P, XTab<T> &X) {
+  int b0[3], nb[3];
+  for (int d = 0; d < 3; d++) {
+    b0[d] = xl_floordiv(a[d], c.bsz[lev][d]);
+    nb[d] = xl_floordiv(b[d], c.bsz[lev][d]) - b0[d] + 1;
+  }
+  const long long ne = (long long)nb[0] * nb[1] * nb[2];
+  __syncthreads();  // the previous patch's table is no longer read
+  if (threadIdx.x == 0) {
+    for (int d = 0; d < 3; d++) {
+      X.b0[d] = b0[d];
+      X.nb[d] = nb[d];
+    }
+    X.ok = ne <= XT;
+  }
+  if (ne <= XT) {
+    for (int e = threadIdx.x; e < (int)ne; e += blockDim.x) {
+      const int bb[3] = {b0[0] + e % nb[0], b0[1] + (e / nb[0]) % nb[1], b0[2] + e / (nb[0] * nb[1])};
+      int w[3];
+      for (int d = 0; d < 3; d++) w[d] = xl_posmod(bb[d], c.mapd[lev][d]);
+      const int Q = c.omap[lev][((long long)w[2] * c.mapd[lev][1] + w[1]) * c.mapd[lev][0] + w[0]];
+      X.A[e] = nullptr;
+      if (Q < 0) continue;  // no patch of the level there (never asked for)
+      T ww[3];
+      const int rc = xl_slices<T>(c, Q, t, X.A[e], X.dB[e], X.dC[e], ww);
+      if (rc) {
+        X.A[e] = nullptr;
+        xl_status(c, rc, P);
+        continue;
+      }
+      for (int d = 0; d < 3; d++) {
+        X.w[d][e] = ww[d];
+        X.n[d][e] = c.geo[Q].n[d];
+        X.lo[d][e] = c.geo[Q].lo[d] + (bb[d] - w[d]) * c.bsz[lev][d];
+      }
+    }
+  }
+  __syncthreads();
+}
 
 // Owner on level lev of the (unwrapped) level-lev cell g, its local cell
 // index, and the slices for time t.  Returns 0, or an error code.
 template <typename T>
-__device__ int xl_source(const DevCtx &c, int lev, const int g[3], double t, XSrc<T> &s) {
+__device__ __forceinline__ int xl_source(const DevCtx &c, int lev, const int g[3], double t, const XTab<T> &X, XSrc<T> &s) {
+  if (X.ok) {
+    int k[3];
+    for (int d = 0; d < 3; d++) k[d] = __float2int_rd(((float)g[d] + 0.5f) * c.binv[lev][d]) - X.b0[d];
+    const int e = (k[2] * X.nb[1] + k[1]) * X.nb[0] + k[0];
+    s.A = X.A[e];
+    if (!s.A) return DSP_ERR_INVALID_ARG;
+    s.B = X.dB[e] ? s.A + X.dB[e] : nullptr;
+    s.C = X.dC[e] ? s.A + X.dC[e] : nullptr;
+    for (int d = 0; d < 3; d++) {
+      s.w[d] = X.w[d][e];
+      s.n[d] = X.n[d][e];
+      s.loc[d] = g[d] - X.lo[d][e];
+    }
+    return DSP_OK;
+  }
   int w[3];
   for (int d = 0; d < 3; d++) w[d] = xl_posmod(g[d], c.L[lev][d]);
   const int Q = c.omap[lev][xl_block(c, lev, w)];
   if (Q < 0) return DSP_ERR_INVALID_ARG;
-  const PatchGeo &gq = c.geo[Q];
-  for (int d = 0; d < 3; d++) s.loc[d] = w[d] - gq.lo[d];
-  s.Q = Q;
-  const T *base = (const T *)c.slab + gq.off;
-  SlicePick pk;
-  if (pick_slices<false>(c, Q, t, pk) != DSP_OK) return DSP_ERR_BRACKET;
-  s.A = base + (long long)pk.s[0] * c.slot_stride;
-  s.B = pk.n >= 2 ? base + (long long)pk.s[1] * c.slot_stride : nullptr;
-  s.C = pk.n == 3 ? base + (long long)pk.s[2] * c.slot_stride : nullptr;
-  for (int q = 0; q < 3; q++) s.w[q] = q < pk.n ? (T)pk.w[q] : T(0);
+  for (int d = 0; d < 3; d++) {
+    s.n[d] = c.geo[Q].n[d];
+    s.loc[d] = w[d] - c.geo[Q].lo[d];
+  }
+  long long dB, dC;
+  const int rc = xl_slices<T>(c, Q, t, s.A, dB, dC, s.w);
+  if (rc) return rc;
+  s.B = dB ? s.A + dB : nullptr;
+  s.C = dC ? s.A + dC : nullptr;
   return DSP_OK;
 }
 
@@ -80,13 +165,12 @@ __device__ __forceinline__ T xl_val(const XSrc<T> &s, long long idx) {
 
 // Conserved values of level-lev cell g at time t.
 template <typename T>
-__device__ int xl_cell(const DevCtx &c, int lev, const int g[3], double t, T u[5]) {
+__device__ __forceinline__ int xl_cell(const DevCtx &c, int lev, const int g[3], double t, const XTab<T> &X, T u[5]) {
   XSrc<T> s;
-  const int rc = xl_source<T>(c, lev, g, t, s);
+  const int rc = xl_source<T>(c, lev, g, t, X, s);
   if (rc) return rc;
-  const PatchGeo &gq = c.geo[s.Q];
-  const long long nc = (long long)gq.n[0] * gq.n[1] * gq.n[2];
-  const long long id = ((long long)s.loc[2] * gq.n[1] + s.loc[1]) * gq.n[0] + s.loc[0];
+  const long long nc = (long long)s.n[0] * s.n[1] * s.n[2];
+  const long long id = ((long long)s.loc[2] * s.n[1] + s.loc[1]) * s.n[0] + s.loc[0];
   for (int q = 0; q < 5; q++) u[q] = xl_val(s, q * nc + id);
   return DSP_OK;
 }
@@ -94,12 +178,11 @@ __device__ int xl_cell(const DevCtx &c, int lev, const int g[3], double t, T u[5
 // Face along ax on the low side of level-lev cell g (up = 1: its high side,
 // owned by the same patch) at time t.
 template <typename T>
-__device__ int xl_face(const DevCtx &c, int lev, int ax, const int g[3], int up, double t, T *out) {
+__device__ __forceinline__ int xl_face(const DevCtx &c, int lev, int ax, const int g[3], int up, double t, const XTab<T> &X, T *out) {
   XSrc<T> s;
-  const int rc = xl_source<T>(c, lev, g, t, s);
+  const int rc = xl_source<T>(c, lev, g, t, X, s);
   if (rc) return rc;
-  const PatchGeo &gq = c.geo[s.Q];
-  const int qx = gq.n[0], qy = gq.n[1], qz = gq.n[2];
+  const int qx = s.n[0], qy = s.n[1], qz = s.n[2];
   s.loc[ax] += up;
   const long long nc = (long long)qx * qy * qz;
   long long idx;
@@ -117,18 +200,17 @@ __device__ int xl_face(const DevCtx &c, int lev, int ax, const int g[3], int up,
 // level-1 patch holds all of them: level-1 patches cover whole level-0
 // cells).
 template <typename T>
-__device__ int xl_restrict_cell(const DevCtx &c, const int C[3], double t, T u[5]) {
+__device__ __forceinline__ int xl_restrict_cell(const DevCtx &c, const int C[3], double t, const XTab<T> &X, T u[5]) {
   const int f0[3] = {2 * C[0], 2 * C[1], 2 * C[2]};
   XSrc<T> s;
-  const int rc = xl_source<T>(c, 1, f0, t, s);
+  const int rc = xl_source<T>(c, 1, f0, t, X, s);
   if (rc) return rc;
-  const PatchGeo &gq = c.geo[s.Q];
-  const long long nc = (long long)gq.n[0] * gq.n[1] * gq.n[2];
+  const long long nc = (long long)s.n[0] * s.n[1] * s.n[2];
   T acc[5] = {T(0), T(0), T(0), T(0), T(0)};
   for (int kz = 0; kz < 2; kz++)
     for (int ky = 0; ky < 2; ky++)
       for (int kx = 0; kx < 2; kx++) {
-        const long long id = ((long long)(s.loc[2] + kz) * gq.n[1] + s.loc[1] + ky) * gq.n[0] + s.loc[0] + kx;
+        const long long id = ((long long)(s.loc[2] + kz) * s.n[1] + s.loc[1] + ky) * s.n[0] + s.loc[0] + kx;
         for (int q = 0; q < 5; q++) acc[q] = acc[q] + xl_val(s, q * nc + id);
       }
   for (int q = 0; q < 5; q++) u[q] = T(0.125) * acc[q];
@@ -138,13 +220,12 @@ __device__ int xl_restrict_cell(const DevCtx &c, const int C[3], double t, T u[5
 // Face along ax on the low side of level-0 cell C, the mean of the 4 level-1
 // faces on it (the children's low faces, in one level-1 patch).
 template <typename T>
-__device__ int xl_restrict_face(const DevCtx &c, int ax, const int C[3], double t, T *out) {
+__device__ __forceinline__ int xl_restrict_face(const DevCtx &c, int ax, const int C[3], double t, const XTab<T> &X, T *out) {
   const int f0[3] = {2 * C[0], 2 * C[1], 2 * C[2]};
   XSrc<T> s;
-  const int rc = xl_source<T>(c, 1, f0, t, s);
+  const int rc = xl_source<T>(c, 1, f0, t, X, s);
   if (rc) return rc;
-  const PatchGeo &gq = c.geo[s.Q];
-  const int qx = gq.n[0], qy = gq.n[1], qz = gq.n[2];
+  const int qx = s.n[0], qy = s.n[1], qz = s.n[2];
   const long long nc = (long long)qx * qy * qz;
   T acc = T(0);
   for (int kz = 0; kz < 2; kz++)
@@ -215,7 +296,7 @@ __device__ __forceinline__ long long xl_shell_count(const int b[3]) {
 // cells per axis whose first cell is P's cell lo-2: cells x in [-2, n+2),
 // faces along an axis at x in [-2, n+2] (relative to lo).
 template <typename T>
-__device__ void fill_cross_level(const DevCtx &c, int P, int part, int parts) {
+__device__ void fill_cross_level(const DevCtx &c, int P, int part, int parts, XTab<T> &X) {
   const long long i0 = (long long)part * blockDim.x + threadIdx.x, istep = (long long)parts * blockDim.x;
   const PatchGeo &gp = c.geo[P];
   const int lev = gp.level;
@@ -244,6 +325,15 @@ __device__ void fill_cross_level(const DevCtx &c, int P, int part, int parts) {
     const int f0 = m[0] + (ax == 0), f1 = m[1] + (ax == 1);
     return fofs[ax] + ((long long)(x[2] + 2) * f1 + (x[1] + 2)) * f0 + (x[0] + 2);
   };
+  {
+    // the other level's cells this patch may take values from
+    int a[3], b[3];
+    for (int d = 0; d < 3; d++) {
+      a[d] = lev == 0 ? 2 * (gp.lo[d] - 2) : xl_floordiv(gp.lo[d] - 2, 2) - 1;
+      b[d] = lev == 0 ? 2 * (gp.lo[d] + n[d] + 2) + 1 : xl_floordiv(gp.lo[d] + n[d] + 2, 2);
+    }
+    xl_table<T>(c, 1 - lev, a, b, t, P, X);
+  }
   if (lev == 0) {
     // restriction: guard cells and faces whose cell is covered by level 1
     // (the guard cells are the 2-deep shell of the (n+4)^3 box)
@@ -256,7 +346,7 @@ __device__ void fill_cross_level(const DevCtx &c, int P, int part, int parts) {
       const int g[3] = {gp.lo[0] + x[0], gp.lo[1] + x[1], gp.lo[2] + x[2]};
       if (!xl_cross(c, 0, g)) continue;
       T u[5];
-      const int rc = xl_restrict_cell<T>(c, g, t, u);
+      const int rc = xl_restrict_cell<T>(c, g, t, X, u);
       if (rc) {
         xl_status(c, rc, P);
         return;
@@ -275,7 +365,7 @@ __device__ void fill_cross_level(const DevCtx &c, int P, int part, int parts) {
         const int g[3] = {gp.lo[0] + x[0], gp.lo[1] + x[1], gp.lo[2] + x[2]};
         if (!xl_cross(c, 0, g)) continue;
         T v;
-        const int rc = xl_restrict_face<T>(c, ax, g, t, &v);
+        const int rc = xl_restrict_face<T>(c, ax, g, t, X, &v);
         if (rc) {
           xl_status(c, rc, P);
           return;
@@ -314,13 +404,13 @@ __device__ void fill_cross_level(const DevCtx &c, int P, int part, int parts) {
     int rc = DSP_OK;
     if (any_cell) {
       T uc[5], ul[5], ur[5], sl[3][5];
-      rc = xl_cell<T>(c, 0, C, t, uc);
+      rc = xl_cell<T>(c, 0, C, t, X, uc);
       for (int d = 0; d < 3 && rc == DSP_OK; d++) {
         int Cm[3] = {C[0], C[1], C[2]}, Cp[3] = {C[0], C[1], C[2]};
         Cm[d] -= 1;
         Cp[d] += 1;
-        rc = xl_cell<T>(c, 0, Cm, t, ul);
-        if (rc == DSP_OK) rc = xl_cell<T>(c, 0, Cp, t, ur);
+        rc = xl_cell<T>(c, 0, Cm, t, X, ul);
+        if (rc == DSP_OK) rc = xl_cell<T>(c, 0, Cp, t, X, ur);
         if (rc == DSP_OK)
           for (int q = 0; q < 5; q++) sl[d][q] = mc(uc[q] - ul[q], ur[q] - uc[q]);
       }
@@ -351,8 +441,8 @@ __device__ void fill_cross_level(const DevCtx &c, int P, int part, int parts) {
       }
       if (!any_face) continue;
       T lo, hi;
-      rc = xl_face<T>(c, 0, ax, C, 0, t, &lo);
-      if (rc == DSP_OK) rc = xl_face<T>(c, 0, ax, C, 1, t, &hi);
+      rc = xl_face<T>(c, 0, ax, C, 0, t, X, &lo);
+      if (rc == DSP_OK) rc = xl_face<T>(c, 0, ax, C, 1, t, X, &hi);
       if (rc) {
         xl_status(c, rc, P);
         return;
@@ -371,11 +461,12 @@ __device__ void fill_cross_level(const DevCtx &c, int P, int part, int parts) {
 constexpr int XL_PARTS = 8;
 template <typename T>
 __global__ void __launch_bounds__(256) xlevel_kernel(DevCtx c) {
+  __shared__ XTab<T> X;
   const int nr = c.ctl[CTL_NREADY];
   for (long long w = blockIdx.x; w < (long long)nr * XL_PARTS; w += gridDim.x) {
     const int P = c.R[w / XL_PARTS];
     if (c.gofs[P] < 0) continue;
-    fill_cross_level<T>(c, P, (int)(w % XL_PARTS), XL_PARTS);
+    fill_cross_level<T>(c, P, (int)(w % XL_PARTS), XL_PARTS, X);
   }
 }
 

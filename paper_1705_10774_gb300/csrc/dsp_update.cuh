@@ -1367,7 +1367,7 @@ __global__ void __launch_bounds__(NT, MINB) queue_kernel(DevCtx c, double t_end)
 }
 template <typename T, int TX, int TY, int NT, int MINB, int VARIANT, int RS, int NI>
 int launch_update(const DevCtx &c, int grid, void *stream, int cls, int cls_end) {
-  // the shared-memory attribute was set by update_grid when the context was
+  // the shared-memory attribute was set by update_slots when the context was
   // created (a launch may be inside a stream capture)
   const size_t smem = update_smem<T, TX, TY, NI>();
   update_kernel<T, TX, TY, NT, MINB, VARIANT, RS, NI><<<grid, NT, smem, (cudaStream_t)stream>>>(c, cls, cls_end);
@@ -1396,6 +1396,8 @@ int launch_queue(const DevCtx &c, int grid, double t_end, void *stream) {
   return cudaGetLastError() == cudaSuccess ? DSP_OK : DSP_ERR_CUDA;
 }
 
+// Blocks of the update kernel that run at once on the current device (and its
+// shared-memory attribute, which a launch inside a stream capture cannot set).
 template <typename T, int TX, int TY, int NT, int MINB, int VARIANT, int RS, int NI>
 int update_slots() {
   const size_t smem = update_smem<T, TX, TY, NI>();
@@ -1405,14 +1407,6 @@ int update_slots() {
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, update_kernel<T, TX, TY, NT, MINB, VARIANT, RS, NI>, NT, smem);
   return nsm * (per < 1 ? 1 : per);
-}
-
-template <typename T, int TX, int TY, int NT, int MINB, int VARIANT, int RS, int NI>
-int update_grid(const DevCtx &c, int cls, int cls_end) {
-  long long maxwork = 0;  // every patch of the classes ready, its z runs cut to single planes
-  for (int k = cls; k < cls_end; k++) maxwork += c.cls_tiles[k] * (c.cls_slots[k] > 0 ? c.cls_tz[k] : 1);
-  const long long g = update_slots<T, TX, TY, NT, MINB, VARIANT, RS, NI>();
-  return (int)(g < maxwork ? g : maxwork);
 }
 
 }  // namespace dsp
