@@ -728,15 +728,16 @@ constexpr int kNumVariants = sizeof(kVariants) / sizeof(kVariants[0]);
 // smallest cost times its number of tiles, so that wide tiles serve patches
 // they divide and 16 x 8 tiles serve the small and the ragged ones.
 double tile_cost(const KernelVariant *v) {
-  if (v->nonideal || v->riemann) return 1.0;
+  if (v->nonideal) return 1.0;
   switch (v->id) {
-    case 1: return 0.66;   // FP64, 8 x 8
-    case 3: return 0.60;   // FP64 with FMA, 8 x 8
-    case 4: return 1.17;   // FP64 with FMA, 16 x 12
-    case 6: return 1.40;   // FP32, 16 x 8, one block per SM
-    case 7: return 1.76;   // FP32, 32 x 8
-    case 8: return 1.94;   // FP32, 16 x 16
-    case 21: return 1.90;  // FP32, 24 x 8 (slower than its share: nine warps, one block per SM)
+    case 1: return 0.65;   // FP64, 8 x 8
+    case 3: return 0.58;   // FP64 with FMA, 8 x 8
+    case 4: return 1.22;   // FP64 with FMA, 16 x 12
+    case 6: return 1.34;   // FP32, 16 x 8, one block per SM
+    case 7: return 1.73;   // FP32, 32 x 8
+    case 8: return 1.89;   // FP32, 16 x 16
+    case 21: return 1.90;  // FP32, 24 x 8 (alone 1.52; its own launch beside the other sizes' costs more)
+    case 22: return 1.73;  // FP32 HLLD, 32 x 8
     default: return 1.0;   // 16 x 8
   }
 }

@@ -68,16 +68,27 @@ struct March {
   static constexpr int QSZ = 65;   // [2]
   static constexpr int QE = 67;    // [3] x-, y- and z-edge EMFs
   static constexpr int QNB = 70;   // [2] new x- and y-faces
-  static constexpr int QB = 72;    // [2] x- and y-faces of the plane to come
-  static constexpr int QU = 74;    // [5] the cell just updated (its own thread's)
-  static constexpr int NQ = 79 + 1;
+  static constexpr int QU = 72;    // [5] the cell just updated, and its old values (its own thread's)
+  // FP32: raw values of the plane to come [rho, m, E, x-, y-face below, z-face
+  // above], copied here asynchronously, the old faces of the update and, where
+  // two blocks need not share an SM, the state at the upper z-face of the
+  // previous plane; FP64 holds these in registers and publishes the two faces
+  static constexpr bool SL = sizeof(T) == 4;
+  static constexpr int QRAW = 78;  // [8]
+  static constexpr int QOF = 86;   // [3]
+  static constexpr int QZP = 90;   // [8]
+  static constexpr bool SZP = SL && !PAIR;
+  static constexpr int QB = SL ? QRAW + 5 : 77;  // [2] x- and y-faces of the plane to come
+  static constexpr int NQ = !SL ? 80 : SZP ? 98 : 90;
   static constexpr int total = (PAIR ? NQ / 2 : NQ) * PLANE;
   // threads: the tile's columns, the halo columns with fluxes (right column,
   // top row), then the other halo columns (bottom row, left column, corners);
   // the ring around the halo (primitives only) is dealt to the halo's threads
   static constexpr int NTILE = TX * TY;
-  static constexpr int HB0 = NTILE + (TX + TY + 31) / 32 * 32;
-  static constexpr int NEED = HB0 + TX + TY + 4;
+  // (from the next warp on, unless packing them saves a warp)
+  static constexpr int NHA = TX + TY, NHB = TX + TY + 4, RND = (NHA + 31) / 32 * 32;
+  static constexpr int HB0 = NTILE + ((RND + NHB + 31) / 32 > (NHA + NHB + 31) / 32 ? NHA : RND);
+  static constexpr int NEED = HB0 + NHB;
   static constexpr int NRING = 2 * (TX + 2) + 2 * (TY + 2);
 };
 
@@ -193,6 +204,8 @@ __device__ __forceinline__ void march_tile(const DevCtx &c, const int P, const d
   const bool xfull = xf && j >= 0 && j < ty, yfull = yf && i >= 0 && i < tx;
   const bool zf = h1 && ((i >= 0 && i < tx) || (j >= 0 && j < ty));
   const bool ez_ = h1 && i >= 0 && j >= 0, ex_ = ez_ && i < tx, ey_ = ez_ && j < ty;
+  // a warp with any flux computes fluxes in all its faces' lanes at once
+  const bool xw = __any_sync(0xffffffffu, xfull), yw = __any_sync(0xffffffffu, yfull);
   const bool ownxy = x >= 0 && x < nx && y >= 0 && y < ny;
   T *const s0p = sm + (j + 2) * PITCH + (i + 2);
   // a column of the ring around the halo (primitives only)
@@ -212,6 +225,7 @@ __device__ __forceinline__ void march_tile(const DevCtx &c, const int P, const d
     }
   }
   const int rx = x0 + ri, ry = y0 + rj;
+  const int edge_ax = !ring ? -1 : ri == tx + 1 ? 0 : rj == ty + 1 ? 1 : -1;
   const bool rown = rx >= 0 && rx < nx && ry >= 0 && ry < ny;
   T *const r0p = sm + (rj + 2) * PITCH + (ri + 2);
 
@@ -224,9 +238,9 @@ __device__ __forceinline__ void march_tile(const DevCtx &c, const int P, const d
     const int ez = __float2int_rd(((float)gz + 0.5f) * binv[2]) - bz0;
     return (ez * nby + ey) * nbx + ex;
   };
-  auto fetch = [&](const T *p, int e) -> T {
+  // a table entry's value: from one slice (bl = 0), or blended from two or three
+  auto value = [&](const T *p, int bl, int e) -> T {
     T a = *src(p);
-    const int bl = S.blend[e];
     if (bl) {
       const T b = *src(p + (long long)(((bl >> 2) & 63) - 16) * c.slot_stride);
       if ((bl & 3) == 2) {
@@ -238,52 +252,123 @@ __device__ __forceinline__ void march_tile(const DevCtx &c, const int P, const d
     }
     return a;
   };
-  // the face along ax on the low side of patch cell (xx, yy, zz): the
-  // patch's own where it lies on one of its interior cells, else that of the
-  // patch that owns the cell
-  auto face = [&](int ax, int xx, int yy, int zz) -> T {
-    const int mx0 = nx + (ax == 0), my0 = ny + (ax == 1), mz0 = nz + (ax == 2);
-    if (xx >= 0 && xx < mx0 && yy >= 0 && yy < my0 && zz >= 0 && zz < mz0)
-      return *src(own + (ax == 0 ? ofx : ax == 1 ? ofy : ofz) + ((long long)zz * my0 + yy) * mx0 + xx);
-    const int gx = lox + xx, gy = loy + yy, gz = loz + zz;
-    const int e = entry(gx, gy, gz);
-    const int mx = S.n[0][e], my = S.n[1][e], mz = S.n[2][e];
-    const int lx = gx - S.lo[0][e], ly = gy - S.lo[1][e], lz = gz - S.lo[2][e];
-    const long long m = (long long)mx * my * mz;
-    long long o = 5 * m;
-    if (ax >= 1) o += (long long)(mx + 1) * my * mz;
-    if (ax == 2) o += (long long)mx * (my + 1) * mz;
-    const int fx = mx + (ax == 0), fy = my + (ax == 1);
-    return fetch(srcA[e] + o + ((long long)lz * fy + ly) * fx + lx, e);
+  // where a value lives: its address in a slice, blend code and table entry
+  struct Loc {
+    const T *p;
+    int bl, e;
   };
-  // the five conserved values of patch cell (xx, yy, q), its low x- and
-  // y-faces and its high z-face
-  auto load_cell = [&](int xx, int yy, bool inxy, int q, T u[5], T &fx, T &fy, T &fz) {
-    if (inxy && q >= 0 && q < nz) {
+  auto get = [&](const Loc &l) -> T { return value(l.p, l.bl, l.e); };
+  // Table entries of a column, its +x and its +y neighbour in the lowest layer
+  // of map blocks (a byte each); the layer of a plane.
+  const int nbxy = nbx * nby;
+  auto layer = [&](int z) -> int { return (__float2int_rd(((float)(loz + z) + 0.5f) * binv[2]) - bz0) * nbxy; };
+  auto entries = [&](int xx, int yy) -> int {
+    return entry(lox + xx, loy + yy, bz0 * bsz[2]) | entry(lox + xx + 1, loy + yy, bz0 * bsz[2]) << 8 |
+           entry(lox + xx, loy + yy + 1, bz0 * bsz[2]) << 16;
+  };
+  // a patch seen from patch cell (xx, yy, zz): the patch itself, or the one of
+  // table entry e (chosen by selects: the halo's warps mix both)
+  struct View {
+    const T *A;
+    int mx, my, mz, lx, ly, lz, bl, e;
+  };
+  auto view = [&](bool mine, int e, int xx, int yy, int zz) -> View {
+    const int4 n = S.nb[e], l = S.lo4[e];
+    View v;
+    v.A = mine ? own : srcA[e];
+    v.mx = mine ? nx : n.x;
+    v.my = mine ? ny : n.y;
+    v.mz = mine ? nz : n.z;
+    v.lx = mine ? xx : lox + xx - l.x;
+    v.ly = mine ? yy : loy + yy - l.y;
+    v.lz = mine ? zz : loz + zz - l.z;
+    v.bl = mine ? 0 : n.w;
+    v.e = e;
+    return v;
+  };
+  // the face along ax on the low side of the view's cell
+  auto face_at = [&](int ax, const View &v) -> Loc {
+    const long long m = (long long)v.mx * v.my * v.mz;
+    long long o = 5 * m;
+    if (ax >= 1) o += (long long)(v.mx + 1) * v.my * v.mz;
+    if (ax == 2) o += (long long)v.mx * (v.my + 1) * v.mz;
+    return {v.A + o + ((long long)v.lz * (v.my + (ax == 1)) + v.ly) * (v.mx + (ax == 0)) + v.lx, v.bl, v.e};
+  };
+  // whether the face along ax on the low side of patch cell (xx, yy, zz) is
+  // the patch's own: it lies on one of its interior cells
+  auto own_face = [&](int ax, int xx, int yy, int zz) -> bool {
+    return xx >= 0 && xx < nx + (ax == 0) && yy >= 0 && yy < ny + (ax == 1) && zz >= 0 && zz < nz + (ax == 2);
+  };
+  // that face: the patch's own, else that of the patch that owns the cell (ent:
+  // the column's table entry in the lowest layer)
+  auto face = [&](int ax, int ent, int xx, int yy, int zz) -> Loc {
+    return face_at(ax, view(own_face(ax, xx, yy, zz), ent + layer(zz), xx, yy, zz));
+  };
+  // Hands to `to` (value number, place) the five conserved values of patch
+  // cell (xx, yy, q), its low x- and y-faces (5, 6) and its high z-face (7);
+  // for a ring column (RING) also its high x- and y-faces and its low z-face.
+  // Straight-line code: with a branch for every own or foreign value, and a
+  // lookup and a blend test for each, the halo's warps took 4800 clocks a
+  // plane here where the tile's took 1350, and every warp waited for them
+  // (3700 now; 256^3 in FP32: 2.87 -> 2.67 ms a sweep).  Addresses kept and
+  // stepped from plane to plane, in shared or in local memory, took longer.
+  auto load_cell = [&](auto rr, int ents, int xx, int yy, bool inxy, int q, auto to) {
+    constexpr bool RING = decltype(rr)::value;
+    const bool zin = q >= 0 && q < nz;
+    if (__all_sync(__activemask(), inxy && zin)) {
       const long long o = ((long long)q * ny + yy) * nx + xx;
       const T *const a = own + o;
 #pragma unroll
-      for (int k = 0; k < 5; k++) u[k] = *src(a + k * nc);
-      fx = *src(a + ofx + ((long long)q * ny + yy));
-      fy = *src(a + ofy + (long long)q * nx);
-      fz = *src(a + ofz + (long long)nx * ny);
+      for (int k = 0; k < 5; k++) to(k, Loc{a + k * nc, 0, 0});
+      const T *const ax = a + ofx + ((long long)q * ny + yy), *const ay = a + ofy + (long long)q * nx, *const az = a + ofz;
+      to(5, Loc{ax, 0, 0});
+      to(6, Loc{ay, 0, 0});
+      to(7, Loc{az + (long long)nx * ny, 0, 0});
+      if constexpr (RING) {
+        to(8, Loc{ax + 1, 0, 0});
+        to(9, Loc{ay + nx, 0, 0});
+        to(10, Loc{az, 0, 0});
+      }
       return;
     }
-    const int gx = lox + xx, gy = loy + yy, gz = loz + q;
-    const int e = entry(gx, gy, gz);
-    const int mx = S.n[0][e], my = S.n[1][e], mz = S.n[2][e];
-    const int lx = gx - S.lo[0][e], ly = gy - S.lo[1][e], lz = gz - S.lo[2][e];
-    const long long m = (long long)mx * my * mz;
-    const long long row = (long long)lz * my + ly;
-    const T *const a = srcA[e] + row * mx + lx;
+    const int ent = (ents & 255), e = ent + layer(q);
+    const View v = view(inxy && zin, e, xx, yy, q);
+    const long long m = (long long)v.mx * v.my * v.mz;
+    const T *const a = v.A + ((long long)v.lz * v.my + v.ly) * v.mx + v.lx;
 #pragma unroll
-    for (int k = 0; k < 5; k++) u[k] = fetch(a + k * m, e);
-    const bool zin = q >= 0 && q < nz;
-    if (zin && xx == nx && yy >= 0 && yy < ny) fx = *src(own + ofx + ((long long)q * ny + yy) * (nx + 1) + nx);
-    else fx = fetch(a + 5 * m + row, e);
-    if (zin && yy == ny && xx >= 0 && xx < nx) fy = *src(own + ofy + ((long long)q * (ny + 1) + ny) * nx + xx);
-    else fy = fetch(a + 5 * m + (long long)(mx + 1) * my * mz + (long long)lz * mx, e);
-    fz = face(2, xx, yy, q + 1);
+    for (int k = 0; k < 5; k++) to(k, Loc{a + k * m, v.bl, e});
+    to(5, face_at(0, view(own_face(0, xx, yy, q), e, xx, yy, q)));
+    to(6, face_at(1, view(own_face(1, xx, yy, q), e, xx, yy, q)));
+    to(7, face(2, ent, xx, yy, q + 1));
+    if constexpr (RING) {
+      to(8, face(0, ents >> 8 & 255, xx + 1, yy, q));
+      to(9, face(1, ents >> 16, xx, yy + 1, q));
+      to(10, face(2, ent, xx, yy, q));
+    }
+  };
+  // The values of load_cell into shared memory, place(k): plain copies are
+  // asynchronous (no register is held, and no branch taken, while they are in
+  // flight); blended ones follow where a lane of the warp has any.  With
+  // concurrent publishers: plain loads.
+  auto stage = [&](auto rr, int ents, int xx, int yy, bool inxy, int q, auto place) {
+    if constexpr (CONC) {
+      load_cell(rr, ents, xx, yy, inxy, q, [&](int k, const Loc &l) { *place(k) = get(l); });
+    } else {
+      int blends = 0;
+      load_cell(rr, ents, xx, yy, inxy, q, [&](int k, const Loc &l) {
+        blends |= l.bl;
+        cp_async_if(place(k), src(l.p), l.bl == 0);
+      });
+      if (__any_sync(__activemask(), blends != 0))
+        load_cell(rr, ents, xx, yy, inxy, q, [&](int k, const Loc &l) {
+          if (l.bl) *place(k) = get(l);
+        });
+    }
+  };
+  auto copy_to = [&](T *d, const Loc &l) {
+    if constexpr (CONC) *d = get(l);
+    else if (l.bl == 0) cp_async_elem(d, src(l.p));
+    else *d = get(l);
   };
   auto prim_of = [&](const T u[5], T fxl, T fxh, T fyl, T fyh, T fzl, T fzh, T W[8], int *floored) {
     if constexpr (kFast) fast::prim(u[0], u[1], u[2], u[3], u[4], fxl, fxh, fyl, fyh, fzl, fzh, gm1, W, floored);
@@ -294,8 +379,11 @@ __device__ __forceinline__ void march_tile(const DevCtx &c, const int P, const d
   auto up = [&](T w, T d) -> T { return kFast ? w + d : w + half * d; };
   auto dn = [&](T w, T d) -> T { return kFast ? w - d : w - half * d; };
 
+  const int ents = entries(x, y), rents = ring ? entries(rx, ry) : 0;
+
   // raw values of the next plane and the z-face below it
-  T ru[5], rfx = T(0), rfy = T(0), rfz = T(0), fzl = T(0);
+  T raw[8];  // FP64 only
+  T fzl = T(0);
   T fd[3], zdl[8];  // plane p's normal-field differences, W(p) - W(p-1)
 
   T smax_t = T(0);
@@ -363,11 +451,15 @@ __device__ __forceinline__ void march_tile(const DevCtx &c, const int P, const d
       T fn[3], w0[8];
       if (it >= -2) {
         const T fxh = s0p[M::q(M::QB) + 1], fyh = s0p[M::q(M::QB + 1) + PITCH];
-        prim_of(ru, rfx, fxh, rfy, fyh, fzl, rfz, wn, nullptr);
-        fn[0] = fxh - rfx;
-        fn[1] = fyh - rfy;
-        fn[2] = rfz - fzl;
-        fzl = rfz;
+        if constexpr (M::SL) {
+#pragma unroll
+          for (int k = 0; k < 8; k++) raw[k] = s0p[M::q(M::QRAW + k)];
+        }
+        prim_of(raw, raw[5], fxh, raw[6], fyh, fzl, raw[7], wn, nullptr);
+        fn[0] = fxh - raw[5];
+        fn[1] = fyh - raw[6];
+        fn[2] = raw[7] - fzl;
+        fzl = raw[7];
       }
       if (it >= -1) {
 #pragma unroll
@@ -409,27 +501,6 @@ __device__ __forceinline__ void march_tile(const DevCtx &c, const int P, const d
 #pragma unroll
           for (int k = 0; k < 8; k++) { dX[k] = T(0); dY[k] = T(0); dZ[k] = T(0); ws[k] = w0[k]; }
         }
-        // face states
-        T XR[8], YR[8], ZR[8], ZU[8];
-#pragma unroll
-        for (int k = 0; k < 8; k++) {
-          XR[k] = up(ws[k], dX[k]);
-          YR[k] = up(ws[k], dY[k]);
-          ZU[k] = up(ws[k], dZ[k]);
-          xr[k] = dn(ws[k], dX[k]);
-          yr[k] = dn(ws[k], dY[k]);
-          ZR[k] = dn(ws[k], dZ[k]);
-          if constexpr (sizeof(T) == 8) {  // held, not added up again for each corner
-            keep(XR[k]);
-            keep(YR[k]);
-            keep(ZU[k]);
-            keep(xr[k]);
-            keep(yr[k]);
-            keep(ZR[k]);
-          }
-          s0p[M::q(M::QXR + k)] = XR[k];
-          s0p[M::q(M::QYR + k)] = YR[k];
-        }
         // corners: a face state of the edge's a axis extrapolated along b
         auto corner = [&](const T *Wa, const T *db, bool bp, int va, int vb, int ba, int bb, T o[3]) {
           auto at = [&](int k) -> T { return bp ? up(Wa[k], db[k]) : dn(Wa[k], db[k]); };
@@ -444,37 +515,61 @@ __device__ __forceinline__ void march_tile(const DevCtx &c, const int P, const d
           for (int k = 0; k < 3; k++) b[M::q(k0 + k)] = o[k];
         };
         T *const bp_ = s0p + par * M::q(M::PSTEP);
-        T o[3];
-        // z-edges: a = x, b = y
-        corner(XR, dY, true, VX, VY, BX, BY, o);
+        T o[3], U_[8], ZR[8];
+        // x-face states, z-edges (a = x, b = y)
+#pragma unroll
+        for (int k = 0; k < 8; k++) {
+          U_[k] = up(ws[k], dX[k]);
+          xr[k] = dn(ws[k], dX[k]);
+          s0p[M::q(M::QXR + k)] = U_[k];
+        }
+        corner(U_, dY, true, VX, VY, BX, BY, o);
         put3(M::QZC, o, s0p);
         corner(xr, dY, true, VX, VY, BX, BY, o);
         put3(M::QZC + 3, o, s0p);
-        corner(XR, dY, false, VX, VY, BX, BY, o);
+        corner(U_, dY, false, VX, VY, BX, BY, o);
         put3(M::QZC + 6, o, s0p);
         corner(xr, dY, false, VX, VY, BX, BY, cz0);
-        // x-edges: a = y, b = z
-        corner(YR, dZ, false, VY, VZ, BY, BZ, o);
+        // y-face states, x-edges (a = y, b = z)
+#pragma unroll
+        for (int k = 0; k < 8; k++) {
+          U_[k] = up(ws[k], dY[k]);
+          yr[k] = dn(ws[k], dY[k]);
+          s0p[M::q(M::QYR + k)] = U_[k];
+        }
+        corner(U_, dZ, false, VY, VZ, BY, BZ, o);
         put3(M::QXM, o, s0p);
-        corner(YR, dZ, true, VY, VZ, BY, BZ, o);
+        corner(U_, dZ, true, VY, VZ, BY, BZ, o);
         put3(M::QXP, o, bp_);
         corner(yr, dZ, true, VY, VZ, BY, BZ, cxn);
         corner(yr, dZ, false, VY, VZ, BY, BZ, cx0);
-        // y-edges: a = z, b = x
+        // z-face states, y-edges (a = z, b = x)
+#pragma unroll
+        for (int k = 0; k < 8; k++) {
+          U_[k] = up(ws[k], dZ[k]);
+          ZR[k] = dn(ws[k], dZ[k]);
+        }
         corner(ZR, dX, true, VZ, VX, BZ, BX, o);
         put3(M::QYM, o, s0p);
-        corner(ZU, dX, true, VZ, VX, BZ, BX, o);
+        corner(U_, dX, true, VZ, VX, BZ, BX, o);
         put3(M::QYP, o, bp_);
-        corner(ZU, dX, false, VZ, VX, BZ, BX, cyn);
+        corner(U_, dX, false, VZ, VX, BZ, BX, cyn);
         corner(ZR, dX, false, VZ, VX, BZ, BX, cy0);
         // the z-face at p-1/2 needs this column alone
         if (it > 0 && zf) {
+          if constexpr (M::SZP) {
+#pragma unroll
+            for (int k = 0; k < 8; k++) zp[k] = s0p[M::q(M::QZP + k)];
+          }
           face_of(std::integral_constant<int, 2>{}, zp, ZR, incol, fz, sz);
           s0p[M::q(M::QSZ)] = sz[0];
           s0p[M::q(M::QSZ + 1)] = sz[1];
         }
 #pragma unroll
-        for (int k = 0; k < 8; k++) zp[k] = ZU[k];
+        for (int k = 0; k < 8; k++) {
+          if constexpr (M::SZP) s0p[M::q(M::QZP + k)] = U_[k];
+          else zp[k] = U_[k];
+        }
       } else if (it == -1) {
 #pragma unroll
         for (int k = 0; k < 8; k++) zdl[k] = wn[k] - w0[k];
@@ -514,7 +609,7 @@ __device__ __forceinline__ void march_tile(const DevCtx &c, const int P, const d
       T L8[8];
 #pragma unroll
       for (int k = 0; k < 8; k++) L8[k] = s0p[M::q(M::QXR + k) - 1];
-      face_of(std::integral_constant<int, 0>{}, L8, xr, xfull && flux, fx, sx);
+      face_of(std::integral_constant<int, 0>{}, L8, xr, xw && flux, fx, sx);
       s0p[M::q(M::QSX)] = sx[0];
       s0p[M::q(M::QSX + 1)] = sx[1];
       if (xfull && flux) {
@@ -526,7 +621,7 @@ __device__ __forceinline__ void march_tile(const DevCtx &c, const int P, const d
       T L8[8];
 #pragma unroll
       for (int k = 0; k < 8; k++) L8[k] = s0p[M::q(M::QYR + k) - PITCH];
-      face_of(std::integral_constant<int, 1>{}, L8, yr, yfull && flux, fy, sy);
+      face_of(std::integral_constant<int, 1>{}, L8, yr, yw && flux, fy, sy);
       s0p[M::q(M::QSY)] = sy[0];
       s0p[M::q(M::QSY + 1)] = sy[1];
       if (yfull && flux) {
@@ -536,34 +631,58 @@ __device__ __forceinline__ void march_tile(const DevCtx &c, const int P, const d
     }
     // loads of plane p+2, of plane p+1 of the ring and of the old values to
     // update: used after the next barrier
-    T ou[5], obx = T(0), oby = T(0), obz = T(0), dun[5];
     const bool upd = it >= 2 && it <= nt_;
     const long long orow = (long long)(p - 1) * ny + y;
+    T dun[5];
+    T ou[5], of[3], ring_raw[11], edge = T(0);  // FP64 only
     if (upd) {
       if (incol) {
+        const T *const a = own + orow * nx + x;
 #pragma unroll
-        for (int k = 0; k < 5; k++) ou[k] = *src(own + k * nc + orow * nx + x);
+        for (int k = 0; k < 5; k++) {
+          if constexpr (M::SL) copy_to(s0p + M::q(M::QU + k), Loc{a + k * nc, 0, 0});
+          else ou[k] = *src(a + k * nc);
+        }
       }
-      if (xfull) obx = *src(own + ofx + orow * (nx + 1) + x);
-      if (yfull) oby = *src(own + ofy + (orow + (p - 1)) * nx + x);
+      if (xfull) {
+        const T *const a = own + ofx + orow * (nx + 1) + x;
+        if constexpr (M::SL) copy_to(s0p + M::q(M::QOF), Loc{a, 0, 0});
+        else of[0] = *src(a);
+      }
+      if (yfull) {
+        const T *const a = own + ofy + (orow + (p - 1)) * nx + x;
+        if constexpr (M::SL) copy_to(s0p + M::q(M::QOF + 1), Loc{a, 0, 0});
+        else of[1] = *src(a);
+      }
     }
-    if (it > 0 && it <= nt_ && incol) obz = *src(own + ofz + (orow + ny) * nx + x);
-    T qu[5], qf[6];
-    T bxe = T(0), bye = T(0);  // the ring's low faces that the halo's columns take as their high ones
+    if (it > 0 && it <= nt_ && incol) {
+      const T *const a = own + ofz + (orow + ny) * nx + x;
+      if constexpr (M::SL) copy_to(s0p + M::q(M::QOF + 2), Loc{a, 0, 0});
+      else of[2] = *src(a);
+    }
     if (h1 && it <= tz) {
-      if (it == -3) fzl = face(2, x, y, p + 2);
-      load_cell(x, y, ownxy, p + 2, ru, rfx, rfy, rfz);
+      if (it == -3) fzl = get(face(2, ents & 255, x, y, p + 2));
+      if constexpr (M::SL)
+        stage(std::false_type{}, ents, x, y, ownxy, p + 2, [&](int k) { return s0p + M::q(M::QRAW + k); });
+      else
+        load_cell(std::false_type{}, ents, x, y, ownxy, p + 2, [&](int k, const Loc &l) { raw[k] = get(l); });
     }
     if (ring) {
+      // (FP32: at the ring's places in planes that only the halo's columns use)
       if (it >= -2 && it <= tz) {
-        load_cell(rx, ry, rown, p + 1, qu, qf[0], qf[2], qf[5]);
-        qf[1] = face(0, rx + 1, ry, p + 1);
-        qf[3] = face(1, rx, ry + 1, p + 1);
-        qf[4] = face(2, rx, ry, p + 1);
+        if constexpr (M::SL)
+          stage(std::true_type{}, rents, rx, ry, rown, p + 1, [&](int k) { return r0p + M::q(M::QXR + k); });
+        else
+          load_cell(std::true_type{}, rents, rx, ry, rown, p + 1, [&](int k, const Loc &l) { ring_raw[k] = get(l); });
       }
-      if (it <= tz && ri == tx + 1) bxe = face(0, rx, ry, p + 2);
-      if (it <= tz && rj == ty + 1) bye = face(1, rx, ry, p + 2);
+      // the low face that a halo column takes as its high one
+      if (it <= tz && edge_ax >= 0) {
+        const Loc l = face(edge_ax, rents & 255, rx, ry, p + 2);
+        if constexpr (M::SL) copy_to(r0p + (edge_ax == 0 ? M::q(M::QB) : M::q(M::QB + 1)), l);
+        else edge = get(l);
+      }
     }
+    if constexpr (M::SL) cp_async_commit();
     __syncthreads();
 
     // ---- 3: edge EMFs and in-plane divergence
@@ -577,6 +696,14 @@ __device__ __forceinline__ void march_tile(const DevCtx &c, const int P, const d
       else return emf(ell, erl, elr, err, all, arl, alr, arr, bll, brl, blr, brr, apa, ama, apb, amb);
     };
     T exn = T(0), eyn = T(0), ezn = T(0);
+    if (it >= 0 && it <= nt_) {  // the column's own speeds, from where phase 2 put them
+#pragma unroll
+      for (int k = 0; k < 2; k++) {
+        sx[k] = s0p[M::q(M::QSX + k)];
+        sy[k] = s0p[M::q(M::QSY + k)];
+        sz[k] = s0p[M::q(M::QSZ + k)];
+      }
+    }
     if (it > 0 && it <= nt_) {
       if (ex_) {
         // LL and LR from the column at -y, RL and RR this column's
@@ -611,7 +738,8 @@ __device__ __forceinline__ void march_tile(const DevCtx &c, const int P, const d
       if (incol && flux) {
 #pragma unroll
         for (int k = 0; k < 5; k++)
-          dun[k] = (s0p[M::q(M::QFX + k) + 1] - fx[k]) + (s0p[M::q(M::QFY + k) + PITCH] - fy[k]);
+          dun[k] = (s0p[M::q(M::QFX + k) + 1] - s0p[M::q(M::QFX + k)]) +
+                   (s0p[M::q(M::QFY + k) + PITCH] - s0p[M::q(M::QFY + k)]);
       }
     }
 #pragma unroll
@@ -624,46 +752,55 @@ __device__ __forceinline__ void march_tile(const DevCtx &c, const int P, const d
       sxp[k] = sx[k];
       syp[k] = sy[k];
     }
+    if constexpr (M::SL) cp_async_wait<0>();
     if (it <= tz) {
-      if (h1) {
-        s0p[M::q(M::QB)] = rfx;
-        s0p[M::q(M::QB + 1)] = rfy;
-      }
-      if (ring) {
-        if (it >= -2) {
-          T W[8];
-          prim_of(qu, qf[0], qf[1], qf[2], qf[3], qf[4], qf[5], W, nullptr);
-#pragma unroll
-          for (int k = 0; k < 8; k++) r0p[M::q(M::QW + k)] = W[k];
+      if constexpr (!M::SL) {
+        if (h1) {
+          s0p[M::q(M::QB)] = raw[5];
+          s0p[M::q(M::QB + 1)] = raw[6];
         }
-        if (ri == tx + 1) r0p[M::q(M::QB)] = bxe;
-        if (rj == ty + 1) r0p[M::q(M::QB + 1)] = bye;
+        if (edge_ax == 0) r0p[M::q(M::QB)] = edge;
+        if (edge_ax == 1) r0p[M::q(M::QB + 1)] = edge;
+      }
+      if (ring && it >= -2) {
+        T W[8];
+        if constexpr (M::SL) {
+#pragma unroll
+          for (int k = 0; k < 11; k++) ring_raw[k] = r0p[M::q(M::QXR + k)];
+        }
+        prim_of(ring_raw, ring_raw[5], ring_raw[8], ring_raw[6], ring_raw[9], ring_raw[10], ring_raw[7], W, nullptr);
+#pragma unroll
+        for (int k = 0; k < 8; k++) r0p[M::q(M::QW + k)] = W[k];
       }
     }
     __syncthreads();
 
     // ---- the update of plane p-1 and of the z-faces at p-1/2
     auto less = [&](T a, T r) -> T { return kFast ? fast::fm(-dtdx, r, a) : a - dtdx * r; };
+    if constexpr (M::SL) {  // copied by this thread
+#pragma unroll
+      for (int k = 0; k < 3; k++) of[k] = s0p[M::q(M::QOF + k)];
+    }
     if (upd) {
       if (xfull) {
-        const T nfx = less(obx, dey - (eyn - eyp_));
+        const T nfx = less(of[0], dey - (eyn - eyp_));
         s0p[M::q(M::QNB)] = nfx;
         put_global(dst + ofx + orow * (nx + 1) + x, nfx);
       }
       if (yfull) {
-        const T nfy = less(oby, (exn - exp_) - dex);
+        const T nfy = less(of[1], (exn - exp_) - dex);
         s0p[M::q(M::QNB + 1)] = nfy;
         put_global(dst + ofy + (orow + (p - 1)) * nx + x, nfy);
       }
     }
     if (it > 0 && it <= nt_ && incol) {
       nfzl = nfzh;
-      nfzh = less(obz, (s0p[M::q(M::QE + 1) + 1] - eyn) - (s0p[M::q(M::QE) + PITCH] - exn));
+      nfzh = less(of[2], (s0p[M::q(M::QE + 1) + 1] - eyn) - (s0p[M::q(M::QE) + PITCH] - exn));
       put_global(dst + ofz + (orow + ny) * nx + x, nfzh);
       if (upd) {
 #pragma unroll
         for (int k = 0; k < 5; k++) {
-          const T un = less(ou[k], du[k] + (fz[k] - fzp[k]));
+          const T un = less(M::SL ? s0p[M::q(M::QU + k)] : ou[k], du[k] + (fz[k] - fzp[k]));
           s0p[M::q(M::QU + k)] = un;
           put_global(dst + k * nc + orow * nx + x, un);
         }

@@ -93,14 +93,21 @@ enum { GATHER_NOW = 0, GATHER_ISSUE = 1, GATHER_BLEND = 2 };
 template <int M>
 using GatherMode = std::integral_constant<int, M>;
 
+// (No memory clobber: what a copy writes is read only after cp_async_wait,
+// which has one; with it, each copy kept the next one's table lookups and
+// addresses from starting.)
 template <typename T>
 __device__ __forceinline__ void cp_async_elem(T *dst, const T *src) {
   static_assert(sizeof(T) == 4 || sizeof(T) == 8, "4- or 8-byte elements");
   const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-  if constexpr (sizeof(T) == 4)
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(src) : "memory");
-  else
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src) : "memory");
+  if constexpr (sizeof(T) == 4) asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(src));
+  else asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src));
+}
+// The copy where `on` holds, without a branch (4-byte elements).
+__device__ __forceinline__ void cp_async_if(float *dst, const float *src, bool on) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %2, 0;\n\t@p cp.async.ca.shared.global [%0], [%1], 4;\n\t}" ::"r"(d),
+               "l"(src), "r"((int)on));
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
@@ -125,10 +132,9 @@ __device__ __forceinline__ void set_error(const DevCtx &c, int code, int P, long
 template <typename T, int NT>
 struct TileShared {
   const T *srcA[TABMAX];
-  int blend[TABMAX];
   T wgt[3][TABMAX];
-  int lo[3][TABMAX];
-  int n[3][TABMAX];
+  int4 nb[TABMAX];  // size (x, y, z) and blend
+  int4 lo4[TABMAX];
   double red[NT / 32];
   int fallback;
   int least;   // FP32 lower bound (bits) on the tile's largest new signal speed
@@ -169,21 +175,13 @@ __device__ __forceinline__ int owner_table(const DevCtx &c, int P, int lev, doub
     if (Q < 0) {
       // the cross-level guard buffer: a patch of n+4 cells at lo-2, in P's
       // own (unwrapped) coordinates
-      for (int d = 0; d < 3; d++) {
-        S.lo[d][e] = gp.lo[d] - 2;
-        S.n[d][e] = gp.n[d] + 4;
-      }
+      S.lo4[e] = make_int4(gp.lo[0] - 2, gp.lo[1] - 2, gp.lo[2] - 2, 0);
+      S.nb[e] = make_int4(gp.n[0] + 4, gp.n[1] + 4, gp.n[2] + 4, 0);
       srcA[e] = (const T *)c.gbuf + c.gofs[P];
-      S.blend[e] = 0;
       continue;
     }
     const PatchGeo &gq = c.geo[Q];
-    S.lo[0][e] = gq.lo[0] + (bx - wx) * bsz[0];
-    S.lo[1][e] = gq.lo[1] + (by - wy) * bsz[1];
-    S.lo[2][e] = gq.lo[2] + (bz - wz) * bsz[2];
-    S.n[0][e] = gq.n[0];
-    S.n[1][e] = gq.n[1];
-    S.n[2][e] = gq.n[2];
+    S.lo4[e] = make_int4(gq.lo[0] + (bx - wx) * bsz[0], gq.lo[1] + (by - wy) * bsz[1], gq.lo[2] + (bz - wz) * bsz[2], 0);
     const T *base = (const T *)c.slab + gq.off;
     SlicePick pk;
     if (pick_slices<CONC>(c, Q, tP, pk) != DSP_OK) {
@@ -197,7 +195,7 @@ __device__ __forceinline__ int owner_table(const DevCtx &c, int P, int lev, doub
       bl = pk.n | ((pk.s[1] - pk.s[0] + 16) << 2) | ((pk.n == 3 ? pk.s[2] - pk.s[0] + 16 : 16) << 8);
       my_blend = 1;
     }
-    S.blend[e] = bl;
+    S.nb[e] = make_int4(gq.n[0], gq.n[1], gq.n[2], bl);
 #pragma unroll
     for (int q = 0; q < 3; q++) S.wgt[q][e] = q < pk.n ? (T)pk.w[q] : T(0);
   }
@@ -309,7 +307,7 @@ __device__ __forceinline__ void process_tile(const DevCtx &c, const int P, const
     const T *p;
     int e;
   };
-  auto blended = [&](const Loc &l) -> bool { return l.e >= 0 && S.blend[l.e] != 0; };
+  auto blended = [&](const Loc &l) -> bool { return l.e >= 0 && S.nb[l.e].w != 0; };
   // Bounds-checked build: every global address of the update is tested
   // against the slab of slices and the cross-level guard buffers; an address
   // outside both records DSP_ERR_BOUNDS and the access is redirected to the
@@ -337,7 +335,7 @@ __device__ __forceinline__ void process_tile(const DevCtx &c, const int P, const
   auto fetch = [&](const Loc &l) -> T {
     T a = *src(l.p);
     if (l.e >= 0) {
-      const int bl = S.blend[l.e];
+      const int bl = S.nb[l.e].w;
       if (bl) {
         const T b = *src(l.p + (long long)(((bl >> 2) & 63) - 16) * c.slot_stride);
         if ((bl & 3) == 2) {
@@ -366,8 +364,8 @@ __device__ __forceinline__ void process_tile(const DevCtx &c, const int P, const
       return {own + q * nc + ((long long)z * ny + y) * nx + x, -1};
     const int gx = lox + x, gy = loy + y, gz = loz + z;
     const int e = entry(gx, gy, gz);
-    const int mx = S.n[0][e], my = S.n[1][e], mz = S.n[2][e];
-    const int lx = gx - S.lo[0][e], ly = gy - S.lo[1][e], lz = gz - S.lo[2][e];
+    const int mx = S.nb[e].x, my = S.nb[e].y, mz = S.nb[e].z;
+    const int lx = gx - S.lo4[e].x, ly = gy - S.lo4[e].y, lz = gz - S.lo4[e].z;
     return {srcA[e] + q * ((long long)mx * my * mz) + ((long long)lz * my + ly) * mx + lx, e};
   };
   // Face below cell (x,y,z) along each axis: the patch's own face when it
@@ -378,8 +376,8 @@ __device__ __forceinline__ void process_tile(const DevCtx &c, const int P, const
       return {own + ofx + ((long long)z * ny + y) * (nx + 1) + x, -1};
     const int gx = lox + x, gy = loy + y, gz = loz + z;
     const int e = entry(gx, gy, gz);
-    const int mx = S.n[0][e], my = S.n[1][e], mz = S.n[2][e];
-    const int lx = gx - S.lo[0][e], ly = gy - S.lo[1][e], lz = gz - S.lo[2][e];
+    const int mx = S.nb[e].x, my = S.nb[e].y, mz = S.nb[e].z;
+    const int lx = gx - S.lo4[e].x, ly = gy - S.lo4[e].y, lz = gz - S.lo4[e].z;
     return {srcA[e] + 5 * ((long long)mx * my * mz) + ((long long)lz * my + ly) * (mx + 1) + lx, e};
   };
   auto facey_loc = [&](int x, int y, int z) -> Loc {
@@ -387,8 +385,8 @@ __device__ __forceinline__ void process_tile(const DevCtx &c, const int P, const
       return {own + ofy + ((long long)z * (ny + 1) + y) * nx + x, -1};
     const int gx = lox + x, gy = loy + y, gz = loz + z;
     const int e = entry(gx, gy, gz);
-    const int mx = S.n[0][e], my = S.n[1][e], mz = S.n[2][e];
-    const int lx = gx - S.lo[0][e], ly = gy - S.lo[1][e], lz = gz - S.lo[2][e];
+    const int mx = S.nb[e].x, my = S.nb[e].y, mz = S.nb[e].z;
+    const int lx = gx - S.lo4[e].x, ly = gy - S.lo4[e].y, lz = gz - S.lo4[e].z;
     const long long m = (long long)mx * my * mz;
     return {srcA[e] + 5 * m + (long long)(mx + 1) * my * mz + ((long long)lz * (my + 1) + ly) * mx + lx, e};
   };
@@ -397,8 +395,8 @@ __device__ __forceinline__ void process_tile(const DevCtx &c, const int P, const
       return {own + ofz + ((long long)z * ny + y) * nx + x, -1};
     const int gx = lox + x, gy = loy + y, gz = loz + z;
     const int e = entry(gx, gy, gz);
-    const int mx = S.n[0][e], my = S.n[1][e], mz = S.n[2][e];
-    const int lx = gx - S.lo[0][e], ly = gy - S.lo[1][e], lz = gz - S.lo[2][e];
+    const int mx = S.nb[e].x, my = S.nb[e].y, mz = S.nb[e].z;
+    const int lx = gx - S.lo4[e].x, ly = gy - S.lo4[e].y, lz = gz - S.lo4[e].z;
     const long long m = (long long)mx * my * mz;
     return {srcA[e] + 5 * m + (long long)(mx + 1) * my * mz + (long long)mx * (my + 1) * mz +
                 ((long long)lz * my + ly) * mx + lx,

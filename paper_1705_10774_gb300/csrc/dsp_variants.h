@@ -20,7 +20,7 @@
   X(4, double, 16, 12, 256, 1, 2, 0, 0)    \
   X(5, float, 16, 8, 192, 2, 1, 0, 0)     \
   X(6, float, 16, 8, 192, 1, 1, 0, 0)     \
-  X(7, float, 32, 8, 384, 1, 1, 0, 0)     \
+  X(7, float, 32, 8, 352, 1, 1, 0, 0)     \
   X(8, float, 16, 16, 352, 1, 1, 0, 0)    \
   X(9, double, 16, 8, 192, 1, 0, 1, 0)    \
   X(10, double, 16, 8, 192, 1, 2, 1, 0)   \
@@ -34,7 +34,8 @@
   X(18, double, 16, 4, 256, 1, 0, 1, 1) \
   X(19, double, 16, 4, 256, 1, 2, 1, 1) \
   X(20, float, 16, 8, 256, 1, 1, 1, 1)   \
-  X(21, float, 24, 8, 288, 1, 1, 0, 0)
+  X(21, float, 24, 8, 288, 1, 1, 0, 0) \
+  X(22, float, 32, 8, 352, 1, 1, 1, 0)
 
 #define DSP_VARIANT_LIST_CHECKED(X)    \
   X(0, double, 16, 8, 192, 1, 0, 0, 0)    \
