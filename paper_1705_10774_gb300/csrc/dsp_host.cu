@@ -728,8 +728,10 @@ constexpr int kNumVariants = sizeof(kVariants) / sizeof(kVariants[0]);
 // smallest cost times its number of tiles, so that wide tiles serve patches
 // they divide and 16 x 8 tiles serve the small and the ragged ones.
 double tile_cost(const KernelVariant *v) {
-  if (v->nonideal) return 1.0;
   switch (v->id) {
+    case 15: return 0.82;  // FP64 with FMA, non-ideal, 16 x 4 with 256 threads (13: 128)
+    case 16: return 0.63;  // FP32, non-ideal, 16 x 4 (14: 16 x 8)
+    case 17: return 0.84;  // FP64, non-ideal, 16 x 4 with 256 threads (12: 128)
     case 1: return 0.65;   // FP64, 8 x 8
     case 3: return 0.58;   // FP64 with FMA, 8 x 8
     case 4: return 1.22;   // FP64 with FMA, 16 x 12
@@ -738,7 +740,7 @@ double tile_cost(const KernelVariant *v) {
     case 8: return 1.89;   // FP32, 16 x 16
     case 21: return 1.90;  // FP32, 24 x 8 (alone 1.52; its own launch beside the other sizes' costs more)
     case 22: return 1.73;  // FP32 HLLD, 32 x 8
-    default: return 1.0;   // 16 x 8
+    default: return 1.0;   // 16 x 8 (non-ideal FP64: 16 x 4)
   }
 }
 

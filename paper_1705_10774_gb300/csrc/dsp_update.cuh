@@ -1,50 +1,58 @@
-// dsp_update.cuh -- the fused per-patch update kernel.
+// dsp_update.cuh -- the fused per-patch update kernel: its work items, the
+// owner table of a tile, the sweep and ready-queue kernels, and the tile
+// update of the variants with non-ideal terms (ideal MHD: dsp_march.cuh).
 //
 // One work item is a tile of one ready patch: TX x TY columns of cells and a
-// run of tz planes along z.  The block marches through the planes; for each
-// plane it
+// run of planes along z.  With non-ideal terms the block marches through the
+// planes phase by phase; for each plane it
 //   A  takes the next plane of the padded tile (radius 2) from the patch's
 //      own newest slice and its neighbours' slices, inter- or extrapolating
 //      in time where a neighbour is not at the patch's time (DISPATCH I,
-//      Sec. 3 A and B), and converts to
-//      primitive variables (the plane's copies were started asynchronously
-//      one plane earlier, so only the time blends remain to compute);
+//      Sec. 3 A and B), and converts to primitive variables (the plane's
+//      copies were started asynchronously one plane earlier, into a ring of
+//      four planes, so only the time blends remain to compute);
 //   B  computes MC-limited slopes and the Hancock half-step predictor;
 //   C  computes HLL (or HLLD) fluxes through the x- and y-faces of the
 //      plane and the z-faces below it;
-//   D  computes the upwind edge EMFs on the x- and y-edges below the plane and
-//      the in-plane part of the flux divergence;
+//   D  computes the upwind edge EMFs on the x- and y-edges below the plane,
+//      with the Ohmic and ambipolar ones (Sec. 4.3), and the in-plane part of
+//      the flux divergence; the Poynting flux of the non-ideal EMFs joins the
+//      energy flux;
 //   E  writes the conservative update of the plane below and the
 //      constrained-transport update of its faces into the patch's next slice
 //      (the oldest slice is overwritten, Sec. 3 A);
 //   F  computes the z-edge EMFs of the plane, the signal speed of the freshly
 //      written cells, and the values carried to the next plane.
-// With the non-ideal terms (NI) phases D and F add the Ohmic and ambipolar
-// EMFs to the edges, and the Poynting flux of those EMFs joins the energy
-// flux before the update of the plane below (DISPATCH I, Sec. 4.3).
 // Every intermediate lives in shared memory; HBM sees the gathered input and
-// the written output only.  The arithmetic per cell, face and edge is the
-// same sequence of operations as the oracle's, so the FP64 build (no FMA
-// contraction) reproduces it bit for bit.
+// the written output only.  Without FMA the arithmetic per cell, face and
+// edge is the same sequence of operations as the oracle's, bit for bit; the
+// other builds take the forms of dsp_fast.cuh.  What bounds it: the FP64 pipe
+// (and latency, at eight warps per SM).  128^3 cells in 32^3 patches, FP64
+// with FMA, Ohmic and ambipolar: 14.6 ms a sweep with synchronous loads and
+// the common forms, 8.9 ms with asynchronous ones, the fast forms, bounded
+// signal speeds and 256 threads.
 #pragma once
 #include <cuda_runtime.h>
 
 #include <type_traits>
 
 #include "dsp_dispatch.cuh"
+#include "dsp_fast.cuh"
 #include "dsp_internal.h"
 #include "dsp_physics.cuh"
 
 namespace dsp {
 
-template <int TX, int TY, int NI = 0>
+// Shared-memory layout of the phase-by-phase tile (non-ideal variants).
+template <int TX, int TY>
 struct Lay {
   static constexpr int H2N = (TX + 4) * (TY + 4);
   static constexpr int H1N = (TX + 2) * (TY + 2);
   static constexpr int FPN = (TX + 5) * (TY + 5);
-  static constexpr int NFB = NI ? 3 : 2;       // face planes held (three for the non-ideal currents)
-  static constexpr int oW = 0;                 // [3 planes][8][H2N] primitive ring
-  static constexpr int oFB = oW + 24 * H2N;    // [NFB planes][4][FPN] faces: x-low, y-low, z-low, z-high
+  // planes held: p-1, p, p+1 (the currents read all three) and the one being copied in
+  static constexpr int NFB = 4;
+  static constexpr int oW = 0;                 // [NFB planes][8][H2N] primitive ring
+  static constexpr int oFB = oW + NFB * 8 * H2N;  // [NFB planes][4][FPN] faces: x-low, y-low, z-low, z-high
   static constexpr int oWS = oFB + NFB * 4 * FPN;  // [8][H1N] predicted state W*
   static constexpr int oDX = oWS + 8 * H1N;    // [8][H1N] slopes along x
   static constexpr int oDY = oDX + 8 * H1N;
@@ -69,20 +77,20 @@ struct Lay {
   // cells, their x- and y-faces, the z-faces below them
   static constexpr int oOLD = oNBZ + 2 * H1N;
   static constexpr int OLDU = 0, OLDX = 5 * TX * TY, OLDY = OLDX + (TX + 1) * TY, OLDZ = OLDY + TX * (TY + 1);
-  // non-ideal terms only: the non-ideal EMFs of the x- and y-edges (two
+  // the non-ideal EMFs of the x- and y-edges (two
   // levels, by parity), of the z-edges of the previous plane, and the ideal
   // energy fluxes of the x- and y-faces of the last two planes (by parity)
   static constexpr int oENX = oOLD + OLDZ + TX * TY;
-  static constexpr int oENY = oENX + (NI ? 2 * H1N : 0);
-  static constexpr int oENZ = oENY + (NI ? 2 * H1N : 0);
-  static constexpr int oFXE = oENZ + (NI ? H1N : 0);
-  static constexpr int oFYE = oFXE + (NI ? 2 * H1N : 0);
+  static constexpr int oENY = oENX + 2 * H1N;
+  static constexpr int oENZ = oENY + 2 * H1N;
+  static constexpr int oFXE = oENZ + H1N;
+  static constexpr int oFYE = oFXE + 2 * H1N;
   // and the edge currents: x- and y-edges of the level below each of two
   // planes, z-edges of two planes (rings by plane parity)
-  static constexpr int oJX = oFYE + (NI ? 2 * H1N : 0);
-  static constexpr int oJY = oJX + (NI ? 2 * H1N : 0);
-  static constexpr int oJZ = oJY + (NI ? 2 * H1N : 0);
-  static constexpr int total = oJZ + (NI ? 2 * H1N : 0);
+  static constexpr int oJX = oFYE + 2 * H1N;
+  static constexpr int oJY = oJX + 2 * H1N;
+  static constexpr int oJZ = oJY + 2 * H1N;
+  static constexpr int total = oJZ + 2 * H1N;
 };
 
 
@@ -219,10 +227,10 @@ template <typename T, int TX, int TY, int NT, bool CONC, int RS, int NI>
 __device__ __forceinline__ void process_tile(const DevCtx &c, const int P, const double dt, const int tile,
                                              const int zlo, const int zrun, T *sm, TileShared<T, NT> &S) {
   static_assert(TX * TY <= NT, "one updated cell per thread");
-  using L = Lay<TX, TY, NI>;
+  using L = Lay<TX, TY>;
   // asynchronous copies of the next plane and of the old values (sweep
-  // dispatcher, ideal MHD)
-  constexpr bool ASYNC = !CONC && !NI;
+  // dispatcher)
+  constexpr bool ASYNC = !CONC;
   // phases C and D as pools of work items over the whole block (FP64), or
   // one loop per axis (FP32)
   constexpr bool POOL = sizeof(T) == 8;
@@ -296,6 +304,7 @@ __device__ __forceinline__ void process_tile(const DevCtx &c, const int P, const
   if (tid == 0) {
     s_fallback = 0;
     S.floors = 0;
+    S.least = 0;
   }
   const int any_blend = __syncthreads_or(my_blend);
 
@@ -409,11 +418,11 @@ __device__ __forceinline__ void process_tile(const DevCtx &c, const int P, const
   // copy (cp.async) of every value that is a plain copy and leaves the
   // blended ones; GATHER_BLEND computes only the blended ones (after the
   // copies have landed).
-  // ring slot of plane q's faces: two planes, or three with non-ideal terms
-  auto fslot = [&](int q) -> int { return NI ? (q - z0 + 3) % 3 : (q - z0 + 2) & 1; };
+  // ring slot of plane q's faces
+  auto fslot = [&](int q) -> int { return (q - z0 + 4) & 3; };
   auto gather_plane = [&](int q, auto mode) {
     constexpr int M = decltype(mode)::value;
-    const int rs = (q - z0 + 3) % 3, fs = fslot(q);
+    const int rs = (q - z0 + 4) & 3, fs = fslot(q);
     T *Wq = Wr + rs * 8 * H2N;
     T *Fq = FB + fs * 4 * FPN;
     auto put = [&](T *dst, const Loc &l) {
@@ -523,7 +532,7 @@ __device__ __forceinline__ void process_tile(const DevCtx &c, const int P, const
     cp_async_commit();
   };
   auto prim_plane = [&](int q) {
-    const int rs = (q - z0 + 3) % 3, fs = fslot(q);
+    const int rs = (q - z0 + 4) & 3, fs = fslot(q);
     T *Wq = Wr + rs * 8 * H2N;
     const T *Fq = FB + fs * 4 * FPN;
     for (int ci = tid; ci < (TX + 4) * (TY + 4); ci += NT) {
@@ -531,8 +540,12 @@ __device__ __forceinline__ void process_tile(const DevCtx &c, const int P, const
       if (i > tx + 1 || j > ty + 1) continue;
       const int h = H2(i, j), f = F5(i, j);
       T Wt[8];
-      prim(Wq[h], Wq[H2N + h], Wq[2 * H2N + h], Wq[3 * H2N + h], Wq[4 * H2N + h], Fq[f], Fq[F5(i + 1, j)],
-           Fq[FPN + f], Fq[FPN + F5(i, j + 1)], Fq[2 * FPN + f], Fq[3 * FPN + f], gamma, Wt);
+      if constexpr (kFast)
+        fast::prim(Wq[h], Wq[H2N + h], Wq[2 * H2N + h], Wq[3 * H2N + h], Wq[4 * H2N + h], Fq[f], Fq[F5(i + 1, j)],
+                   Fq[FPN + f], Fq[FPN + F5(i, j + 1)], Fq[2 * FPN + f], Fq[3 * FPN + f], gamma - T(1), Wt);
+      else
+        prim(Wq[h], Wq[H2N + h], Wq[2 * H2N + h], Wq[3 * H2N + h], Wq[4 * H2N + h], Fq[f], Fq[F5(i + 1, j)],
+             Fq[FPN + f], Fq[FPN + F5(i, j + 1)], Fq[2 * FPN + f], Fq[3 * FPN + f], gamma, Wt);
 #pragma unroll
       for (int k = 0; k < 8; k++) Wq[k * H2N + h] = Wt[k];
     }
@@ -555,8 +568,11 @@ __device__ __forceinline__ void process_tile(const DevCtx &c, const int P, const
   // components the means of the four nearest edges of their own axes.
   const T idx = (T)(1.0 / dxl);
   const T eta_t = (T)c.eta, gad_t = (T)c.gad, rhoi_t = (T)c.rhoi;
+  // the step limits of Eqs. 4 and 8 as signal speeds, in FP32: Ohmic, and
+  // ambipolar per B^2 / rho
+  const float ohm32 = (float)(c.cfl * c.eta / (c.cohm * dxl)), amb32 = c.gad > 0.0 ? (float)(c.cfl / (c.cad * c.gad * c.rhoi * dxl)) : 0.f;
   auto fpl = [&](int q) -> const T * { return FB + fslot(q) * 4 * FPN; };
-  auto wpl = [&](int q) -> const T * { return Wr + ((q - z0 + 3) % 3) * 8 * H2N; };
+  auto wpl = [&](int q) -> const T * { return Wr + ((q - z0 + 4) & 3) * 8 * H2N; };
   auto fxq = [&](int i, int j, int q) -> T { return fpl(q)[F5(i, j)]; };
   auto fyq = [&](int i, int j, int q) -> T { return fpl(q)[FPN + F5(i, j)]; };
   auto fzq = [&](int i, int j, int q) -> T { return fpl(q)[2 * FPN + F5(i, j)]; };
@@ -635,6 +651,12 @@ __device__ __forceinline__ void process_tile(const DevCtx &c, const int P, const
   T *const FXE = sm + L::oFXE;
   T *const FYE = sm + L::oFYE;
 
+  auto emf_of = [&](T ell, T erl, T elr, T err, T all, T arl, T alr, T arr, T bll, T brl, T blr, T brr, T apa, T ama, T apb,
+                    T amb) -> T {
+    if constexpr (kFast)
+      return fast::emf(ell, erl, elr, err, all, arl, alr, arr, bll, brl, blr, brr, apa, ama, apb, amb);
+    else return emf(ell, erl, elr, err, all, arl, alr, arr, bll, brl, blr, brr, apa, ama, apb, amb);
+  };
   T smax_t = T(0);
   T unew[5];
   for (int it = 0; it <= tz + 1; it++) {
@@ -660,12 +682,12 @@ __device__ __forceinline__ void process_tile(const DevCtx &c, const int P, const
     }
     __syncthreads();
     prim_plane(p + 1);
-    if constexpr (NI != 0) currents(p + 1);
+    currents(p + 1);
     __syncthreads();
 
     // ---- B: slopes and predictor on the H1 region of plane p
     {
-      const int rm = (p - 1 - z0 + 3) % 3, r0 = (p - z0 + 3) % 3, rp = (p + 1 - z0 + 3) % 3;
+      const int rm = (p - 1 - z0 + 4) & 3, r0 = (p - z0 + 4) & 3, rp = (p + 1 - z0 + 4) & 3;
       const T *Wm = Wr + rm * 8 * H2N, *W0 = Wr + r0 * 8 * H2N, *Wp = Wr + rp * 8 * H2N;
       const T *F0 = FB + fslot(p) * 4 * FPN;
       for (int ci = tid; ci < (TX + 2) * (TY + 2); ci += NT) {
@@ -684,15 +706,11 @@ __device__ __forceinline__ void process_tile(const DevCtx &c, const int P, const
           if (k == BZ) dZ[k] = F0[3 * FPN + F5(i, j)] - F0[2 * FPN + F5(i, j)];
           else dZ[k] = mc(w8[k] - Wm[k * H2N + h], Wp[k * H2N + h] - w8[k]);
         }
-        predict(w8, dX, dY, dZ, gamma, hdt, ws);
-        bool bad = false;
-#pragma unroll
-        for (int d = 0; d < 3; d++) {
-          const T *d3 = d == 0 ? dX : d == 1 ? dY : dZ;
-          const T rp_ = ws[RHO] + half * d3[RHO], rm_ = ws[RHO] - half * d3[RHO];
-          const T pp_ = ws[PR] + half * d3[PR], pm_ = ws[PR] - half * d3[PR];
-          if (!tpos(rp_) || !tpos(rm_) || !tpos(pp_) || !tpos(pm_)) bad = true;
-        }
+        // (whole slopes: half of dt/dx in place of dt/dx)
+        if constexpr (kFast) fast::predict(w8, dX, dY, dZ, gamma, hdt, ws);
+        else predict(w8, dX, dY, dZ, gamma, hdt, ws);
+        const T dr = fmax_mag(fmax_mag(dX[RHO], dY[RHO]), dZ[RHO]), dp = fmax_mag(fmax_mag(dX[PR], dY[PR]), dZ[PR]);
+        const bool bad = !tpos(ws[RHO] - half * dr) || !tpos(ws[PR] - half * dp);
         if (bad) {
           // once for whole z runs, whatever their parts
           if ((p >= z0 || zlo == 0) && (p < z0 + tz || z0 + tz == zend)) atomicAdd(&s_fallback, 1);
@@ -710,8 +728,8 @@ __device__ __forceinline__ void process_tile(const DevCtx &c, const int P, const
       }
     }
     __syncthreads();
-    // plane p-1's primitive ring slot and plane p's faces are dead now: start
-    // the copies of plane p+2 into them, to land while C..F run
+    // plane p-2's ring slots are dead: start the copies of plane p+2 into
+    // them, to land while C..F run
     if (ASYNC) {
       if (p + 2 <= z0 + tz + 1) gather_plane(p + 2, GatherMode<GATHER_ISSUE>{});
       else cp_async_commit();  // an empty group keeps the wait counts in step
@@ -748,7 +766,8 @@ __device__ __forceinline__ void process_tile(const DevCtx &c, const int P, const
           WR[k] = Sws[o + hr] - half * Sd[o + hr];
         }
         if (full) {
-          face_flux<T, 0, RS>(WL, WR, gamma, igm1, F, SL, SR);
+          if constexpr (kFast && RS == 0) fast::hll(WL, WR, gamma, igm1, F, SL, SR);
+          else face_flux<T, 0, RS>(WL, WR, gamma, igm1, F, SL, SR);
           T *const Fd = d == 0 ? FX : d == 1 ? FY : FZc;
           Fd[hr] = F[0];
           Fd[(1 + d) * H1N + hr] = F[1];
@@ -756,7 +775,8 @@ __device__ __forceinline__ void process_tile(const DevCtx &c, const int P, const
           Fd[(1 + t2) * H1N + hr] = F[3];
           Fd[4 * H1N + hr] = F[4];
         } else {
-          hll_speeds<T, 0>(WL, WR, gamma, SL, SR);
+          if constexpr (kFast && RS == 0) fast::speeds(WL, WR, gamma, SL, SR);
+          else hll_speeds<T, 0>(WL, WR, gamma, SL, SR);
         }
         T *const Sp = d == 0 ? SXc : d == 1 ? SYc : SZ;
         Sp[hr] = SL;
@@ -863,7 +883,7 @@ __device__ __forceinline__ void process_tile(const DevCtx &c, const int P, const
       // with non-ideal terms the energy part waits for the Poynting flux,
       // which needs the edges above this plane: keep the ideal energy
       // fluxes of the plane's x- and y-faces instead
-      constexpr int KD = NI ? 4 : 5;
+      constexpr int KD = 4;
       const bool div = p < z0 + tz;
       auto div_item = [&](int k) {
         const int i = k % TX, j = k / TX;
@@ -914,7 +934,7 @@ __device__ __forceinline__ void process_tile(const DevCtx &c, const int P, const
         const T apz = pmax0(SZ[H1N + hm], SZ[H1N + h0]), amz = nmax0(SZ[hm], SZ[h0]);
         const T apa = d == 0 ? ap2 : apz, ama = d == 0 ? am2 : amz;
         const T apb = d == 0 ? apz : ap2, amb = d == 0 ? amz : am2;
-        T e = emf(Ell, Erl, Elr, E0, Ba_ll, Ba_rl, Ba_lr, ba0, Bb_ll, Bb_rl, Bb_lr, bb0, apa, ama, apb, amb);
+        T e = emf_of(Ell, Erl, Elr, E0, Ba_ll, Ba_rl, Ba_lr, ba0, Bb_ll, Bb_rl, Bb_lr, bb0, apa, ama, apb, amb);
         if constexpr (NI != 0) {
           const T en = d == 0 ? eni_x(i, j, p) : eni_y(i, j, p);
           (d == 0 ? ENX : ENY)[par * H1N + h0] = en;
@@ -935,7 +955,7 @@ __device__ __forceinline__ void process_tile(const DevCtx &c, const int P, const
         if (div)
           for (int ci = tid; ci < TX * TY; ci += NT) div_item(ci);
       }
-      if constexpr (NI != 0) {
+      {
         if (div) {
           for (int ci = tid; ci < (TX + 1) * (TY + 1); ci += NT) {
             const int i = ci % (TX + 1), j = ci / (TX + 1), h = H1(i, j);
@@ -1034,18 +1054,53 @@ __device__ __forceinline__ void process_tile(const DevCtx &c, const int P, const
     __syncthreads();
 
     // ---- F: signal speed of plane p-1, z-edge EMFs of plane p, carried values
-    if (upd && mine) {
+    // (only their maximum counts: FP64 bounds each in FP32 and evaluates
+    // those that may exceed the largest lower bound so far)
+    bool eval = upd && mine;
+    if constexpr (sizeof(T) == 8) {
+      if (upd && tid < (TX * TY + 31) / 32 * 32) {
+        float above = 0.f, below = 0.f;
+        if (eval) {
+          const int h = H1(ui, uj);
+          fast::signal_bounds(unew, NBX[h], NBX[H1(ui + 1, uj)], NBY[h], NBY[H1(ui, uj + 1)], NBZp[h], NBZc[h],
+                              (float)gamma, above, below);
+          // the non-ideal step limits as signal speeds, each to a few roundings
+          float ni = c.eta > 0.0 ? ohm32 : 0.f;
+          if (c.gad > 0.0) {
+            auto mean2 = [](double l, double r) {
+              const float b = 0.5f * (fast::trunc32(l) + fast::trunc32(r));
+              return b * b;
+            };
+            ni = fmaxf(ni, amb32 * (mean2(NBX[h], NBX[H1(ui + 1, uj)]) + mean2(NBY[h], NBY[H1(ui, uj + 1)]) + mean2(NBZp[h], NBZc[h])) /
+                               fast::trunc32(unew[0]));
+          }
+          if (!(ni < 1e18f)) above = __int_as_float(0x7f800000);
+          above = fmaxf(above, ni * 1.00002f);
+          if (below > 0.f) below = fmaxf(below, ni * 0.99998f);
+        }
+        const int w = __reduce_max_sync(0xffffffffu, __float_as_int(fmaxf(below, 0.f)));
+        const int least = max(w, *(volatile int *)&S.least);
+        if ((tid & 31) == 0 && w == least) atomicMax(&S.least, w);
+        eval = eval && !(above < __int_as_float(least));
+      }
+    }
+    if (eval) {
       const int i = ui, j = uj, h = H1(i, j);
       T Wn[8];
       int floored = 0;
-      prim(unew[0], unew[1], unew[2], unew[3], unew[4], NBX[h], NBX[H1(i + 1, j)], NBY[h], NBY[H1(i, j + 1)],
-           NBZp[h], NBZc[h], gamma, Wn, &floored);
+      if constexpr (kFast)
+        fast::prim(unew[0], unew[1], unew[2], unew[3], unew[4], NBX[h], NBX[H1(i + 1, j)], NBY[h], NBY[H1(i, j + 1)],
+                   NBZp[h], NBZc[h], gamma - T(1), Wn, &floored);
+      else
+        prim(unew[0], unew[1], unew[2], unew[3], unew[4], NBX[h], NBX[H1(i + 1, j)], NBY[h], NBY[H1(i, j + 1)],
+             NBZp[h], NBZc[h], gamma, Wn, &floored);
       if (floored) atomicAdd(&S.floors, 1);
       if (!(Wn[RHO] > T(0)) || !(Wn[PR] > T(0)))
         set_error(c, DSP_ERR_UNPHYSICAL, P, ((long long)(p - 1) * ny + (y0 + j)) * nx + (x0 + i));
-      if constexpr (NI != 0)
-        smax_t = tmax(smax_t, tmax(signal_sum(Wn, gamma), nonideal_speed(Wn, c.cfl, c.eta, c.gad, c.rhoi, c.cohm, c.cad, dxl)));
-      else smax_t = tmax(smax_t, signal_sum(Wn, gamma));
+      T sig;
+      if constexpr (kFast) sig = fast::signal_sum(Wn, gamma);
+      else sig = signal_sum(Wn, gamma);
+      smax_t = tmax(smax_t, tmax(sig, nonideal_speed(Wn, c.cfl, c.eta, c.gad, c.rhoi, c.cohm, c.cad, dxl)));
     }
     {
       // the z-edge EMFs of plane p and the values of plane p carried to the
@@ -1085,7 +1140,7 @@ __device__ __forceinline__ void process_tile(const DevCtx &c, const int P, const
         const T ama = nmax0(SXc[hrl], SXc[hrr]);
         const T apb = pmax0(SYc[H1N + hlr], SYc[H1N + hrr]);
         const T amb = nmax0(SYc[hlr], SYc[hrr]);
-        T ez = emf(Ell, Erl, Elr, Err, ll_bx, rl_bx, lr_bx, rr_bx, ll_by, rl_by, lr_by, rr_by, apa, ama, apb, amb);
+        T ez = emf_of(Ell, Erl, Elr, Err, ll_bx, rl_bx, lr_bx, rr_bx, ll_by, rl_by, lr_by, rr_by, apa, ama, apb, amb);
         if constexpr (NI != 0) {
           const T en = eni_z(i, j, p);
           ENZ[hrr] = en;
@@ -1182,7 +1237,7 @@ __device__ __forceinline__ void update_tile(const DevCtx &c, int P, double dt, i
 // its shared memory in bytes
 template <typename T, int TX, int TY, int NI>
 constexpr size_t update_smem() {
-  if constexpr (NI != 0) return sizeof(T) * (size_t)Lay<TX, TY, NI>::total;
+  if constexpr (NI != 0) return sizeof(T) * (size_t)Lay<TX, TY>::total;
   else return sizeof(T) * (size_t)March<T, TX, TY>::total;
 }
 
