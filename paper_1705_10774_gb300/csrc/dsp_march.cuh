@@ -79,7 +79,12 @@ struct March {
   static constexpr int QZP = 90;   // [8]
   static constexpr bool SZP = SL && !PAIR;
   static constexpr int QB = SL ? QRAW + 5 : 77;  // [2] x- and y-faces of the plane to come
-  static constexpr int NQ = !SL ? 80 : SZP ? 98 : 90;
+  static constexpr int NQ1 = !SL ? 80 : SZP ? 98 : 90;
+  // tiles that have an SM to themselves: the second slice's values of a column
+  // blended in time, copied like the first's
+  static constexpr bool DB = SL && (PAIR ? NQ1 / 2 : NQ1) * PLANE * sizeof(T) > 110000;
+  static constexpr int QRB = NQ1;  // [8] (a ring column's: its places from QXR + 11 on)
+  static constexpr int NQ = NQ1 + (DB ? 8 : 0);
   static constexpr int total = (PAIR ? NQ / 2 : NQ) * PLANE;
   // threads: the tile's columns, the halo columns with fluxes (right column,
   // top row), then the other halo columns (bottom row, left column, corners);
@@ -133,13 +138,13 @@ __device__ __forceinline__ void march_tile(const DevCtx &c, const int P, const d
   const int nbx = floordiv(lox + x0 + tx + 2, bsz[0]) - bx0 + 1;
   const int nby = floordiv(loy + y0 + ty + 2, bsz[1]) - by0 + 1;
   const int nbz = floordiv(loz + z0 + tz + 2, bsz[2]) - bz0 + 1;
-  owner_table<T, NT, CONC>(c, P, lev, tP, bx0, by0, bz0, nbx, nby, nbz, S);
+  const int my_blend = owner_table<T, NT, CONC>(c, P, lev, tP, bx0, by0, bz0, nbx, nby, nbz, S);
   if (tid == 0) {
     S.fallback = 0;
     S.floors = 0;
     S.least = 0;
   }
-  __syncthreads();
+  const int any_blend = __syncthreads_or(my_blend);  // some neighbour is not at the patch's time
 
   // Bounds-checked build: every global address of the update is tested
   // against the slab of slices and the cross-level guard buffers; an address
@@ -348,21 +353,48 @@ __device__ __forceinline__ void march_tile(const DevCtx &c, const int P, const d
   };
   // The values of load_cell into shared memory, place(k): plain copies are
   // asynchronous (no register is held, and no branch taken, while they are in
-  // flight); blended ones follow where a lane of the warp has any.  With
-  // concurrent publishers: plain loads.
-  auto stage = [&](auto rr, int ents, int xx, int yy, bool inxy, int q, auto place) {
+  // flight).  Values blended from two slices: both are copied, the second to
+  // second(k), and the thread blends them once they have arrived (bits of the
+  // result: which values; entry e of value k in byte k < 7 or 10: 0, 7: 1, 8:
+  // 2, 9: 3 of `es`); waiting for each in turn took a third of a pass of
+  // local steps on 256^3 (51.0 ms, now 35.2).  Without room for that, and with
+  // three slices, they are loaded here.  With concurrent publishers: plain loads.
+  auto stage = [&](auto rr, int ents, int xx, int yy, bool inxy, int q, auto place, auto second, int &es) -> int {
+    int mask = 0;
     if constexpr (CONC) {
       load_cell(rr, ents, xx, yy, inxy, q, [&](int k, const Loc &l) { *place(k) = get(l); });
+    } else if (!any_blend) {
+      load_cell(rr, ents, xx, yy, inxy, q, [&](int k, const Loc &l) { cp_async_elem(place(k), src(l.p)); });
     } else {
-      int blends = 0;
+      int late = 0;
+      es = 0;
       load_cell(rr, ents, xx, yy, inxy, q, [&](int k, const Loc &l) {
-        blends |= l.bl;
-        cp_async_if(place(k), src(l.p), l.bl == 0);
+        const bool two = M::DB && (l.bl & 3) == 2;
+        cp_async_if(place(k), src(l.p), l.bl == 0 || two);
+        if constexpr (M::DB) {
+          cp_async_if(second(k), src(l.p + (long long)(two ? (l.bl >> 2 & 63) - 16 : 0) * c.slot_stride), two);
+          mask |= two ? 1 << k : 0;
+          if (k == 0 || (k >= 7 && k < 10)) es |= l.e << (k == 0 ? 0 : 8 * (k - 6));
+        }
+        late |= l.bl != 0 && !two;
       });
-      if (__any_sync(__activemask(), blends != 0))
+      if (__any_sync(__activemask(), late))
         load_cell(rr, ents, xx, yy, inxy, q, [&](int k, const Loc &l) {
-          if (l.bl) *place(k) = get(l);
+          if (l.bl && !(M::DB && (l.bl & 3) == 2)) *place(k) = get(l);
         });
+    }
+    return mask;
+  };
+  auto blend = [&](auto nk, int mask, int es, auto place, auto second) {
+    if constexpr (M::DB && !CONC) {
+      constexpr int NK = decltype(nk)::value;
+      if (mask) {
+#pragma unroll
+        for (int k = 0; k < NK; k++) {
+          const T a = *place(k), w = S.wgt[0][es >> (k >= 7 && k < 10 ? 8 * (k - 6) : 0) & 255];
+          if (mask >> k & 1) *place(k) = a + w * (*second(k) - a);
+        }
+      }
     }
   };
   auto copy_to = [&](T *d, const Loc &l) {
@@ -380,6 +412,13 @@ __device__ __forceinline__ void march_tile(const DevCtx &c, const int P, const d
   auto dn = [&](T w, T d) -> T { return kFast ? w - d : w - half * d; };
 
   const int ents = entries(x, y), rents = ring ? entries(rx, ry) : 0;
+
+  // places of the column's and the ring column's values (a ring column's in
+  // planes that only the halo's columns use)
+  auto raw_at = [&](int k) { return s0p + M::q(M::QRAW + k); };
+  auto raw2_at = [&](int k) { return s0p + M::q(M::QRB + k); };
+  auto ring_at = [&](int k) { return r0p + M::q(M::QXR + k); };
+  auto ring2_at = [&](int k) { return r0p + M::q(M::QXR + 11 + k); };
 
   // raw values of the next plane and the z-face below it
   T raw[8];  // FP64 only
@@ -633,6 +672,7 @@ __device__ __forceinline__ void march_tile(const DevCtx &c, const int P, const d
     // update: used after the next barrier
     const bool upd = it >= 2 && it <= nt_;
     const long long orow = (long long)(p - 1) * ny + y;
+    int hm = 0, rm = 0, hes = 0, res = 0, ee = -1;  // blended values on their way
     T dun[5];
     T ou[5], of[3], ring_raw[11], edge = T(0);  // FP64 only
     if (upd) {
@@ -663,7 +703,7 @@ __device__ __forceinline__ void march_tile(const DevCtx &c, const int P, const d
     if (h1 && it <= tz) {
       if (it == -3) fzl = get(face(2, ents & 255, x, y, p + 2));
       if constexpr (M::SL)
-        stage(std::false_type{}, ents, x, y, ownxy, p + 2, [&](int k) { return s0p + M::q(M::QRAW + k); });
+        hm = stage(std::false_type{}, ents, x, y, ownxy, p + 2, raw_at, raw2_at, hes);
       else
         load_cell(std::false_type{}, ents, x, y, ownxy, p + 2, [&](int k, const Loc &l) { raw[k] = get(l); });
     }
@@ -671,15 +711,25 @@ __device__ __forceinline__ void march_tile(const DevCtx &c, const int P, const d
       // (FP32: at the ring's places in planes that only the halo's columns use)
       if (it >= -2 && it <= tz) {
         if constexpr (M::SL)
-          stage(std::true_type{}, rents, rx, ry, rown, p + 1, [&](int k) { return r0p + M::q(M::QXR + k); });
+          rm = stage(std::true_type{}, rents, rx, ry, rown, p + 1, ring_at, ring2_at, res);
         else
           load_cell(std::true_type{}, rents, rx, ry, rown, p + 1, [&](int k, const Loc &l) { ring_raw[k] = get(l); });
       }
       // the low face that a halo column takes as its high one
       if (it <= tz && edge_ax >= 0) {
         const Loc l = face(edge_ax, rents & 255, rx, ry, p + 2);
-        if constexpr (M::SL) copy_to(r0p + (edge_ax == 0 ? M::q(M::QB) : M::q(M::QB + 1)), l);
-        else edge = get(l);
+        if constexpr (M::SL) {
+          T *const d = r0p + (edge_ax == 0 ? M::q(M::QB) : M::q(M::QB + 1));
+          if (M::DB && !CONC && (l.bl & 3) == 2) {
+            cp_async_elem(d, src(l.p));
+            cp_async_elem(r0p + M::q(M::QRB), src(l.p + (long long)((l.bl >> 2 & 63) - 16) * c.slot_stride));
+            ee = l.e;
+          } else {
+            copy_to(d, l);
+          }
+        } else {
+          edge = get(l);
+        }
       }
     }
     if constexpr (M::SL) cp_async_commit();
@@ -753,6 +803,14 @@ __device__ __forceinline__ void march_tile(const DevCtx &c, const int P, const d
       syp[k] = sy[k];
     }
     if constexpr (M::SL) cp_async_wait<0>();
+    if (it <= tz) {
+      if (h1) blend(std::integral_constant<int, 8>{}, hm, hes, raw_at, raw2_at);
+      if (ring) blend(std::integral_constant<int, 11>{}, rm, res, ring_at, ring2_at);
+      if (M::DB && !CONC && ee >= 0) {
+        T *const d = r0p + (edge_ax == 0 ? M::q(M::QB) : M::q(M::QB + 1));
+        *d = *d + S.wgt[0][ee] * (r0p[M::q(M::QRB)] - *d);
+      }
+    }
     if (it <= tz) {
       if constexpr (!M::SL) {
         if (h1) {

@@ -9,7 +9,7 @@
 // variants of one precision, solver and physics compute bit-identical
 // results; they differ only in how the work is spread over threads, so
 // dsp_autotune may pick any of them.  The bounds-checked build
-// (DSP_BOUNDS_CHECK) compiles the three rows of DSP_VARIANT_LIST_CHECKED only.
+// (DSP_BOUNDS_CHECK) compiles the four rows of DSP_VARIANT_LIST_CHECKED only.
 #pragma once
 
 #define DSP_VARIANT_LIST_ALL(X)        \
@@ -40,7 +40,8 @@
 #define DSP_VARIANT_LIST_CHECKED(X)    \
   X(0, double, 16, 8, 192, 1, 0, 0, 0)    \
   X(2, double, 16, 8, 192, 1, 2, 0, 0)    \
-  X(5, float, 16, 8, 192, 2, 1, 0, 0)
+  X(5, float, 16, 8, 192, 2, 1, 0, 0)     \
+  X(7, float, 32, 8, 352, 1, 1, 0, 0)
 
 #ifdef DSP_BOUNDS_CHECK
 #define DSP_VARIANT_LIST(X) DSP_VARIANT_LIST_CHECKED(X)

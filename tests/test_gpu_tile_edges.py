@@ -21,8 +21,8 @@ from oracle import Oracle
 SIZES = [(4, 4, 4), (7, 8, 5), (16, 11, 4), (17, 9, 6), (15, 12, 7), (33, 13, 5), (31, 17, 4), (24, 8, 9), (49, 4, 4)]
 
 
-def _case(n, seed):
-    lay = ics.cartesian((2, 2, 2), n)
+def _case(n, seed, patches=(2, 2, 2)):
+    lay = ics.cartesian(patches, n)
     X, Y, Z = lay.base_cells
     rng = np.random.default_rng(seed)
     shape = (Z, Y, X)
@@ -63,3 +63,32 @@ def test_every_tile_shape_at_its_edges(n, precision):
         tol = 1e-11 if precision == 2 else 1e-5
         assert max(float(np.max(np.abs(a - b))) for a, b in zip(first[0], ref)) <= tol * scale
         assert np.max(np.abs(first[1] - speed)) <= tol * np.max(speed)
+
+
+@pytest.mark.parametrize("riemann", [0, 1])
+@pytest.mark.parametrize("order,grace", [(1, 0.0), (1, 0.4), (2, 0.0)])
+@pytest.mark.parametrize("n", [(33, 9, 5), (16, 8, 8), (7, 20, 4)])
+def test_fp32_tiles_blend_neighbours_alike(n, order, grace, riemann):
+    """FP32 under local steps: the tiles that blend a neighbour's two slices
+    after both have arrived give the bits of those that wait for each value
+    (the 16 x 8 tiles, and every tile where three slices are blended)."""
+    lay, state = _case(n, 3 * sum(n), (4, 2, 2))
+    u = state[0].copy()
+    off = 0
+    for P, (nx, ny, nz) in enumerate(lay.n.astype(int)):  # a hot patch: steps spread over a factor
+        c = nx * ny * nz
+        u[off + 4 * c:off + 5 * c] += 300.0 if P == 0 else 0.0
+        off += 5 * c
+    first = None
+    for vid in [v[0] for v in B.variants() if v[6] == 1 and v[7] == riemann and v[8] == 0]:
+        g = Dispatch(lay.n, lay.lo, precision=1, variant=vid, riemann=riemann, time_mode=1, time_order=order,
+                     grace=grace, nslices=5, gamma=5.0 / 3.0, cfl=0.3, base_cells=lay.base_cells, box_len=lay.box_len,
+                     sched_capacity=4096)
+        g.set_state(*[u] + list(state[1:]))
+        g.advance(max_sweeps=12)
+        out = list(g.get_state()) + list(g.times()) + list(g.schedule())
+        g.close()
+        first = first or out
+        assert len(np.unique(out[-1])) >= 2  # several step sizes, so times differ
+        for a, b in zip(out, first):
+            assert np.array_equal(a, b), vid
