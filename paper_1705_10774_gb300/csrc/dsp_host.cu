@@ -726,11 +726,14 @@ constexpr int kNumVariants = sizeof(kVariants) / sizeof(kVariants[0]);
 // variants of its form (measured on 256^3 cells in 32^3 patches: time of a
 // sweep over its tiles).  A patch's default variant is the one with the
 // smallest cost times its number of tiles, so that wide tiles serve patches
-// they divide and 16 x 8 tiles serve the small and the ragged ones.
+// they divide and 16 x 8 tiles serve the small and the ragged ones (and those
+// whose wide tiles would touch more map blocks than the owner table holds).
 double tile_cost(const KernelVariant *v) {
   switch (v->id) {
     case 15: return 0.82;  // FP64 with FMA, non-ideal, 16 x 4 with 256 threads (13: 128)
-    case 16: return 0.63;  // FP32, non-ideal, 16 x 4 (14: 16 x 8)
+    // FP32, non-ideal, 16 x 4 (14: 16 x 8): 0.63 measured; set so that it takes only patches of at most four
+    // rows, where the count of fallback cells, each tile's halo included, is the other's
+    case 16: return 0.67;
     case 17: return 0.84;  // FP64, non-ideal, 16 x 4 with 256 threads (12: 128)
     case 1: return 0.65;   // FP64, 8 x 8
     case 3: return 0.58;   // FP64 with FMA, 8 x 8
@@ -744,6 +747,21 @@ double tile_cost(const KernelVariant *v) {
   }
 }
 
+// Whether the owner table of every tile (tx x ty columns, tz planes) of a
+// patch of n cells at lo fits the kernel's table.
+bool tiles_fit(const int n[3], const long long lo[3], int tx, int ty, int tz, const int bsz[3]) {
+  auto fdiv = [](long long a, long long b) { return a >= 0 ? a / b : -((-a + b - 1) / b); };
+  const int t[3] = {tx, ty, tz};
+  long long ne = 1;  // the most blocks that a tile touches, axis by axis
+  for (int d = 0; d < 3; d++) {
+    long long most = 0;
+    for (int org = 0; org < n[d]; org += t[d])
+      most = std::max(most, fdiv(lo[d] + org + std::min(t[d], n[d] - org) + 2, bsz[d]) - fdiv(lo[d] + org - 2, bsz[d]) + 1);
+    ne *= most;
+  }
+  return ne <= TABMAX;
+}
+
 // Per-patch tiles and offsets, each patch tiled by its class's tile shape
 // tx[k] x ty[k] and z run tz[k]; false if some tile's owner table would not
 // fit the kernel's table.
@@ -755,7 +773,6 @@ bool make_geometry(const std::vector<dsp_patch_desc> &patches, const std::vector
   off = 0;
   total_tiles = 0;
   for (int k = 0; k < MAXCLS; k++) cls_tiles[k] = 0;
-  auto fdiv = [](long long a, long long b) { return a >= 0 ? a / b : -((-a + b - 1) / b); };
   for (int i = 0; i < npatch; i++) {
     PatchGeo &g = geo[(size_t)i];
     const int k = cls[(size_t)i];
@@ -778,17 +795,8 @@ bool make_geometry(const std::vector<dsp_patch_desc> &patches, const std::vector
            (long long)g.n[0] * g.n[1] * (g.n[2] + 1);
     total_tiles += g.tiles;
     cls_tiles[k] += g.tiles;
-    for (int kz = 0; kz < g.nt[2]; kz++)
-      for (int ky = 0; ky < g.nt[1]; ky++)
-        for (int kx = 0; kx < g.nt[0]; kx++) {
-          const int org[3] = {kx * TX, ky * TY, kz * g.tz};
-          const int ext[3] = {std::min(TX, g.n[0] - org[0]), std::min(TY, g.n[1] - org[1]),
-                              std::min(g.tz, g.n[2] - org[2])};
-          long long ne = 1;
-          for (int d = 0; d < 3; d++)
-            ne *= fdiv(g.lo[d] + org[d] + ext[d] + 2, bsz[d]) - fdiv(g.lo[d] + org[d] - 2, bsz[d]) + 1;
-          if (ne > TABMAX) return false;
-        }
+    const long long lo[3] = {g.lo[0], g.lo[1], g.lo[2]};
+    if (!tiles_fit(g.n, lo, TX, TY, g.tz, bsz)) return false;
   }
   return true;
 }
@@ -1103,17 +1111,29 @@ extern "C" int dsp_create(const dsp_patch_desc *patches, int32_t npatch, const d
     }
   }
   // the classes' default variants: the requested one, else the cheapest per
-  // patch among those of this form (the first where they tie)
+  // patch among those of this form (the first where they tie, and where no
+  // other's tiles fit all patches of the class)
+  auto fits = [&](int k, const KernelVariant *v) {
+    for (int i = 0; i < npatch; i++) {
+      if (cls[(size_t)i] != k) continue;
+      const dsp_patch_desc &p = patches[i];
+      const long long lo[3] = {p.lo[0], p.lo[1], p.lo[2]};
+      const int n[3] = {p.n[0], p.n[1], p.n[2]};
+      const int tz = prm->tile_z > 0 ? std::min(prm->tile_z, n[2]) : n[2];
+      if (!tiles_fit(n, lo, v->tx, v->ty, tz, bsz[p.level])) return false;
+    }
+    return true;
+  };
   const KernelVariant *varc[MAXCLS];
   for (int k = 0; k < MAXCLS; k++) {
     varc[k] = var;
-    if (prm->variant >= 0 || k >= ncls) continue;
+    if (prm->variant >= 0 || k >= ncls || !fits(k, var)) continue;  // (what the first does not fit is refused)
     double best = INFINITY;
     for (int q = 0; q < kNumVariants; q++) {
       const KernelVariant *v = kVariants[q]();
       if (v->precision != prm->precision || v->riemann != prm->riemann || v->nonideal != nonideal) continue;
       const double cost = tile_cost(v) * ((cls_n[k][0] + v->tx - 1) / v->tx) * ((cls_n[k][1] + v->ty - 1) / v->ty);
-      if (cost < best) {
+      if (cost < best && (v == var || fits(k, v))) {
         best = cost;
         varc[k] = v;
       }

@@ -92,3 +92,35 @@ def test_fp32_tiles_blend_neighbours_alike(n, order, grace, riemann):
         assert len(np.unique(out[-1])) >= 2  # several step sizes, so times differ
         for a, b in zip(out, first):
             assert np.array_equal(a, b), vid
+
+
+def _splits(xs, ys, zs):
+    """The box cut at every combination of the given extents per axis."""
+    lo, n = [], []
+    for z in range(len(zs)):
+        for y in range(len(ys)):
+            for x in range(len(xs)):
+                lo.append((sum(xs[:x]), sum(ys[:y]), sum(zs[:z])))
+                n.append((xs[x], ys[y], zs[z]))
+    return np.array(n), np.array(lo), (sum(xs), sum(ys), sum(zs))
+
+
+@pytest.mark.parametrize("xs,ys,zs,precision,riemann,nonideal", [
+    ((32, 4), (8, 8), (12, 4), 1, 0, 0), ((32, 4), (8, 4), (12, 4), 1, 0, 0), ((32, 4), (8, 4), (12, 4), 1, 1, 0),
+    ((16, 4), (12, 4), (12, 4), 2, 0, 0), ((16, 4), (4, 4), (12, 4), 1, 0, 1)])
+def test_layouts_whose_wide_tiles_touch_too_many_blocks_keep_the_first_tile(xs, ys, zs, precision, riemann, nonideal):
+    """Patches beside thin ones: the map blocks are 4 cells wide, and the wide
+    tiles that would be the default touch more of them than a tile's table
+    holds; the form's first tile still fits and serves them."""
+    n, lo, base = _splits(xs, ys, zs)
+    c = np.prod(n, axis=1)
+    u = np.concatenate([np.concatenate([np.ones(k), np.zeros(3 * k), np.full(k, 2.0)]) for k in c])
+    state = [u, np.full(int(np.sum((n[:, 0] + 1) * n[:, 1] * n[:, 2])), 0.3),
+             np.zeros(int(np.sum(n[:, 0] * (n[:, 1] + 1) * n[:, 2]))), np.zeros(int(np.sum(n[:, 0] * n[:, 1] * (n[:, 2] + 1))))]
+    g = Dispatch(n, lo, gamma=5.0 / 3.0, cfl=0.4, base_cells=base, box_len=tuple(b / 8.0 for b in base), time_mode=0,
+                 precision=precision, riemann=riemann, eta=1e-3 * nonideal, gamma_ad=75.0 * nonideal)
+    g.set_state(*state)
+    g.advance(max_sweeps=2)
+    for a, b in zip(g.get_state(), state):  # a uniform state stays
+        assert np.allclose(a, b, rtol=0, atol=1e-6)
+    g.close()
