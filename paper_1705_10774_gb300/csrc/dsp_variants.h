@@ -4,12 +4,18 @@
 // reads this list): id, element type, tile TX x TY, threads per block,
 // minimum resident blocks per SM, precision code of dsp_params (0 FP64
 // without FMA, 1 FP32, 2 FP64 with FMA), Riemann solver of the face fluxes
-// (0 HLL, 1 HLLD), non-ideal terms (1: the Ohmic and ambipolar EMFs; these
-// hold a third plane of faces, so the FP64 rows use a smaller tile).  All
-// variants of one precision, solver and physics compute bit-identical
-// results; they differ only in how the work is spread over threads, so
-// dsp_autotune may pick any of them.  The bounds-checked build
-// (DSP_BOUNDS_CHECK) compiles the four rows of DSP_VARIANT_LIST_CHECKED only.
+// (0 HLL, 1 HLLD), non-ideal terms (1: the Ohmic and ambipolar EMFs).
+// Ideal MHD has a thread per column of the tile and its halo, so the tile
+// sets the block; wide tiles have less halo per cell (256^3 sweeps: FP64 with
+// FMA 36.3 ms for 16 x 12, 41.5 for 16 x 8, 48 for 8 x 8; FP32 2.55 ms for
+// 32 x 8, 2.75 for 16 x 16, 3.2 for two blocks of 16 x 8), small ones fit
+// small patches.  The registers of a column (255 in FP64, 168 in FP32) set how
+// many warps an SM holds.  The non-ideal tiles hold four planes of faces in
+// shared memory, so the FP64 rows use a smaller one.  All variants of one
+// precision, solver and physics compute bit-identical results; they differ
+// only in how the work is spread over threads, so dsp_autotune may pick any of
+// them.  The bounds-checked build (DSP_BOUNDS_CHECK) compiles the three rows
+// of DSP_VARIANT_LIST_CHECKED only.
 #pragma once
 
 #define DSP_VARIANT_LIST_ALL(X)        \
@@ -40,8 +46,7 @@
 #define DSP_VARIANT_LIST_CHECKED(X)    \
   X(0, double, 16, 8, 192, 1, 0, 0, 0)    \
   X(2, double, 16, 8, 192, 1, 2, 0, 0)    \
-  X(5, float, 16, 8, 192, 2, 1, 0, 0)     \
-  X(7, float, 32, 8, 352, 1, 1, 0, 0)
+  X(5, float, 16, 8, 192, 2, 1, 0, 0)
 
 #ifdef DSP_BOUNDS_CHECK
 #define DSP_VARIANT_LIST(X) DSP_VARIANT_LIST_CHECKED(X)
