@@ -1,8 +1,10 @@
 """Build libdispatch_gpu.so in-tree with nvcc for sm_103a.
 
-The FP64 translation units are compiled with -fmad=false (each product and
-sum rounded on its own, as in the FP64 oracle); the FP32 update kernel keeps
-fused multiply-adds.
+The host unit and the kernels that follow the FP64 oracle bit for bit are
+compiled with -fmad=false (each product and sum rounded on its own).  So are
+the other ideal-MHD kernels, which write their fused multiply-adds out and
+thereby round alike for every tile shape; the non-ideal ones of FP64 with
+fused multiply-adds and of FP32 leave contraction to the compiler.
 """
 from __future__ import annotations
 

@@ -74,23 +74,15 @@ __device__ __forceinline__ bool tneg(T a) {
   const typename B::I m = mag_bits(a);
   return B::of(a) < 0 && m != 0 && m <= B::INF;
 }
-// min(a, b) for a, b >= +0 or NaN (as fmin: a NaN operand yields the other)
-template <typename T>
-__device__ __forceinline__ T tmin_nonneg(T a, T b) {
-  using B = FBits<T>;
-  return B::of(a) <= B::of(b) ? a : b;
-}
 // Evaluation order of the update's arithmetic.  kFast = false: the FP64
 // oracle's order, operation for operation (the FMA-free FP64 build).  kFast =
-// true in the builds held to a tolerance rather than bit equality; every
-// kFast form below applies to FP64 only (the FP64 build with fused
-// multiply-adds), where the FP64 pipe is the kernel's bottleneck and the
-// integer units are idle: FP64 comparisons, minima, maxima and power-of-two
-// scalings as integer operations on the bit patterns, one division per edge
-// EMF instead of three, reciprocals and square roots by Newton steps from the
-// hardware approximations.  The FP32 build keeps the plain forms.  Each
-// translation unit of an update-kernel variant defines DSP_FAST_ORDER from
-// its precision.
+// true in the builds held to a tolerance rather than bit equality, FP64 with
+// fused multiply-adds and FP32: they take the forms of dsp_fast.cuh, and from
+// this file the limiter, the HLLD solver and what both share.  In FP64, whose
+// pipe is the kernel's bottleneck, comparisons, minima and maxima are then
+// integer operations on the bit patterns, and reciprocals and square roots
+// Newton steps from the hardware approximations.  Each translation unit of an
+// update-kernel variant defines DSP_FAST_ORDER from its precision.
 #ifndef DSP_FAST_ORDER
 #define DSP_FAST_ORDER 0
 #endif
@@ -135,22 +127,6 @@ __device__ __forceinline__ T nmax0(T a, T b) {
     return tmax(T(0), tmax(-a, -b));
   }
 }
-// a >= 0 and a <= 0 (non-NaN a)
-template <typename T>
-__device__ __forceinline__ bool ge0(T a) {
-  if constexpr (kFast && sizeof(T) == 8) {
-    const long long i = __double_as_longlong(a);
-    return i >= 0 || i == (long long)0x8000000000000000ull;
-  } else {
-    return a >= T(0);
-  }
-}
-template <typename T>
-__device__ __forceinline__ bool le0(T a) {
-  if constexpr (kFast && sizeof(T) == 8) return __double_as_longlong(a) <= 0;
-  else return a <= T(0);
-}
-
 __device__ __forceinline__ double tsqrt(double a) { return sqrt(a); }
 __device__ __forceinline__ float tsqrt(float a) { return sqrtf(a); }
 
@@ -216,7 +192,7 @@ __device__ __forceinline__ T quot(T a, T b) {
 template <typename T>
 __device__ __forceinline__ void prim(T rho, T mx, T my, T mz, T E, T bxl, T bxr, T byl, T byr, T bzl, T bzr,
                                      T gamma, T W[8], int *floored = nullptr) {
-  T irho = rcp_k(rho);
+  T irho = T(1) / rho;
   const T h = T(0.5);
   T Bx = h * (bxl + bxr);
   T By = h * (byl + byr);
@@ -228,15 +204,8 @@ __device__ __forceinline__ void prim(T rho, T mx, T my, T mz, T E, T bxl, T bxr,
   T me = h * (Bx * Bx + By * By + Bz * Bz);
   T p = (gamma - T(1)) * (E - ke - me);
   const T pf = T(PFLOOR) * rho;
-  if constexpr (kFast && sizeof(T) == 8) {
-    // pf > 0: p's bit pattern orders below pf's exactly when p < pf
-    const bool fl = __double_as_longlong(p) < __double_as_longlong(pf);
-    if (floored) *floored = fl;
-    p = fl ? pf : p;
-  } else {
-    if (floored) *floored = p < pf;
-    p = tmax(p, pf);
-  }
+  if (floored) *floored = p < pf;
+  p = tmax(p, pf);
   W[RHO] = rho; W[VX] = vx; W[VY] = vy; W[VZ] = vz; W[PR] = p;
   W[BX] = Bx; W[BY] = By; W[BZ] = Bz;
 }
@@ -274,7 +243,7 @@ __device__ __forceinline__ T nonideal_speed(const T W[8], double cfl, double eta
 // Sum over axes of |v_d| + c_f,d: the signal speed that sets the Courant step.
 template <typename T>
 __device__ __forceinline__ T signal_sum(const T W[8], T gamma) {
-  T ir = rcp_k(W[RHO]);
+  T ir = T(1) / W[RHO];
   T cx = cfast(gamma, ir, W[PR], W[BX], W[BY], W[BZ]);
   T cy = cfast(gamma, ir, W[PR], W[BY], W[BZ], W[BX]);
   T cz = cfast(gamma, ir, W[PR], W[BZ], W[BX], W[BY]);
@@ -344,7 +313,7 @@ __device__ __forceinline__ void predict(const T W[8], const T dX[8], const T dY[
                                         T Ws[8]) {
   T rho = W[RHO], vx = W[VX], vy = W[VY], vz = W[VZ], p = W[PR];
   T Bx = W[BX], By = W[BY], Bz = W[BZ];
-  T irho = rcp_k(rho);
+  T irho = T(1) / rho;
   T divv = dX[VX] + dY[VY] + dZ[VZ];
   T r_rho = -(vx * dX[RHO] + vy * dY[RHO] + vz * dZ[RHO]) - rho * divv;
   T gpx = dX[PR] + (Bx * dX[BX] + By * dX[BY] + Bz * dX[BZ]);
@@ -391,7 +360,7 @@ __device__ __forceinline__ void hll(const T WL[8], const T WR[8], T gamma, T igm
     T E = p * igm1 + h * rho * v2 + h * B2;
     T PT = p + h * B2;
     T vB = vn * bn + vt1 * bt1 + vt2 * bt2;
-    T cf = cfast(gamma, rcp_k(rho), p, bn, bt1, bt2);
+    T cf = cfast(gamma, T(1) / rho, p, bn, bt1, bt2);
     T *Us = side ? UR : UL;
     T *Fs = side ? FR : FL;
     Us[0] = rho; Us[1] = rho * vn; Us[2] = rho * vt1; Us[3] = rho * vt2; Us[4] = E;
@@ -402,11 +371,11 @@ __device__ __forceinline__ void hll(const T WL[8], const T WR[8], T gamma, T igm
     Fs[4] = (E + PT) * vn - bn * vB;
     if (side) { cR = cf; vnR = vn; } else { cL = cf; vnL = vn; }
   }
-  SL = fmin_k(vnL - cL, vnR - cR);
-  SR = fmax_k(vnL + cL, vnR + cR);
+  SL = tmin(vnL - cL, vnR - cR);
+  SR = tmax(vnL + cL, vnR + cR);
   T Fr[5];
-  const T inv = rcp_k(SR - SL);
-  const bool left = ge0(SL), right = le0(SR);
+  const T inv = T(1) / (SR - SL);
+  const bool left = SL >= T(0), right = SR <= T(0);
 #pragma unroll
   for (int q = 0; q < 5; q++) {
     if (left) Fr[q] = FL[q];
@@ -566,17 +535,8 @@ __device__ __forceinline__ T emf(T Ell, T Erl, T Elr, T Err, T Ba_ll, T Ba_rl, T
   T BaL = h * (Ba_ll + Ba_rl);
   T BaR = h * (Ba_lr + Ba_rr);
   T num = apa * apb * Ell + ama * apb * Erl + apa * amb * Elr + ama * amb * Err;
-  if constexpr (kFast && sizeof(T) == 8) {
-    // one reciprocal of the product of the two weight sums serves all three
-    // quotients (FP64: a division costs about five FP64-pipe slots; the FP32
-    // build divides approximately, at the cost of a multiply)
-    const T sa = apa + ama, sb = apb + amb;
-    const T r = rcp_k(sa * sb);
-    return num * r + (apa * ama * sb * r) * (BbR - BbL) - (apb * amb * sa * r) * (BaR - BaL);
-  } else {
-    T den = (apa + ama) * (apb + amb);
-    return num / den + apa * ama / (apa + ama) * (BbR - BbL) - apb * amb / (apb + amb) * (BaR - BaL);
-  }
+  T den = (apa + ama) * (apb + amb);
+  return num / den + apa * ama / (apa + ama) * (BbR - BbL) - apb * amb / (apb + amb) * (BaR - BaL);
 }
 
 }  // namespace dsp
