@@ -366,12 +366,13 @@ __device__ __forceinline__ void march_tile(const DevCtx &c, const int P, const d
   // result: which values; entry e of value k in byte k < 7 or 10: 0, 7: 1, 8:
   // 2, 9: 3 of `es`); waiting for each in turn took a third of a pass of
   // local steps on 256^3 (51.0 ms, now 35.2).  Without room for that, and with
-  // three slices, they are loaded here.  With concurrent publishers: plain loads.
+  // three slices, they are loaded here.  The ready queue copies too: the
+  // slices a tile reads were published before its ticket, and none of them is
+  // overwritten while the patch is behind (216 patches of 32^3 with local
+  // steps: 25.5 ms with plain loads, one waiting for the other, now 13.1).
   auto stage = [&](auto rr, int ents, int xx, int yy, bool inxy, int q, auto place, auto second, int &es) -> int {
     int mask = 0;
-    if constexpr (CONC) {
-      load_cell(rr, ents, xx, yy, inxy, q, [&](int k, const Loc &l) { *place(k) = get(l); });
-    } else if (!any_blend) {
+    if (!any_blend) {
       load_cell(rr, ents, xx, yy, inxy, q, [&](int k, const Loc &l) { cp_async_elem(place(k), src(l.p)); });
     } else {
       int late = 0;
@@ -394,7 +395,7 @@ __device__ __forceinline__ void march_tile(const DevCtx &c, const int P, const d
     return mask;
   };
   auto blend = [&](auto nk, int mask, int es, auto place, auto second) {
-    if constexpr (M::DB && !CONC) {
+    if constexpr (M::DB) {
       constexpr int NK = decltype(nk)::value;
       if (mask) {
 #pragma unroll
@@ -406,8 +407,7 @@ __device__ __forceinline__ void march_tile(const DevCtx &c, const int P, const d
     }
   };
   auto copy_to = [&](T *d, const Loc &l) {
-    if constexpr (CONC) *d = get(l);
-    else if (l.bl == 0) cp_async_elem(d, src(l.p));
+    if (l.bl == 0) cp_async_elem(d, src(l.p));
     else *d = get(l);
   };
   auto prim_of = [&](const T u[5], T fxl, T fxh, T fyl, T fyh, T fzl, T fzh, T W[8], int *floored) {
@@ -728,7 +728,7 @@ __device__ __forceinline__ void march_tile(const DevCtx &c, const int P, const d
         const Loc l = face(edge_ax, rents & 255, rx, ry, p + 2);
         if constexpr (M::SL) {
           T *const d = r0p + (edge_ax == 0 ? M::q(M::QB) : M::q(M::QB + 1));
-          if (M::DB && !CONC && (l.bl & 3) == 2) {
+          if (M::DB && (l.bl & 3) == 2) {
             cp_async_elem(d, src(l.p));
             cp_async_elem(r0p + M::q(M::QRB), src(l.p + (long long)((l.bl >> 2 & 63) - 16) * c.slot_stride));
             ee = l.e;
@@ -814,7 +814,7 @@ __device__ __forceinline__ void march_tile(const DevCtx &c, const int P, const d
     if (it <= tz) {
       if (h1) blend(std::integral_constant<int, 8>{}, hm, hes, raw_at, raw2_at);
       if (ring) blend(std::integral_constant<int, 11>{}, rm, res, ring_at, ring2_at);
-      if (M::DB && !CONC && ee >= 0) {
+      if (M::DB && ee >= 0) {
         T *const d = r0p + (edge_ax == 0 ? M::q(M::QB) : M::q(M::QB + 1));
         *d = *d + S.wgt[0][ee] * (r0p[M::q(M::QRB)] - *d);
       }

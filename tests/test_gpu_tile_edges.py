@@ -124,3 +124,27 @@ def test_layouts_whose_wide_tiles_touch_too_many_blocks_keep_the_first_tile(xs, 
     for a, b in zip(g.get_state(), state):  # a uniform state stays
         assert np.allclose(a, b, rtol=0, atol=1e-6)
     g.close()
+
+
+@pytest.mark.parametrize("riemann", [0, 1])
+@pytest.mark.parametrize("n", [(33, 9, 5), (16, 8, 8), (7, 20, 4)])
+def test_fp32_ready_queue_tiles_end_as_the_sweeps_do(n, riemann):
+    """FP32 under local steps: every tile of the ready-queue kernel, whose
+    copies and blends run beside publishing neighbours, ends in the sweeps' bits."""
+    lay, state = _case(n, 3 * sum(n), (4, 2, 2))
+    u, c = state[0].copy(), int(np.prod(n))
+    u[4 * c:5 * c] += 300.0
+    t_end = 0.05 * lay.dx
+    first = None
+    ids = [v[0] for v in B.variants() if v[6] == 1 and v[7] == riemann and v[8] == 0]
+    for dispatcher, vid in [(1, -1)] + [(0, v) for v in ids + [-1]]:
+        g = Dispatch(lay.n, lay.lo, precision=1, variant=vid, riemann=riemann, time_mode=1, dispatcher=dispatcher,
+                     gamma=5.0 / 3.0, cfl=0.3, base_cells=lay.base_cells, box_len=lay.box_len)
+        g.set_state(*[u] + list(state[1:]))
+        st = g.advance(t_end=t_end)
+        out = list(g.get_state()) + [g.times()[0]]
+        g.close()
+        assert st["patch_updates"] > lay.npatch
+        first = first or out
+        for a, b in zip(out, first):
+            assert np.array_equal(a, b), (dispatcher, vid)
