@@ -732,9 +732,11 @@ constexpr int kNumVariants = sizeof(kVariants) / sizeof(kVariants[0]);
 // slice of a blend, wait for each blended value: ready queue, FP32, 16^3 patches
 // 12.6 ms against 9.2 for 16 x 16, 32^3 20.9 against 12.9 for 32 x 8, 13 x 21 x
 // 17 13.3 against 10.1 for 16 x 16 (which global steps would tile by 16 x 8).
-double tile_cost(const KernelVariant *v, bool local) {
+// In the queue they lose on patches of one tile too (8^3 13.8 ms against 11.6
+// for 24 x 8, 6 x 7 x 5 7.4 against 6.6): there they count more than any.
+double tile_cost(const KernelVariant *v, bool local, bool queue) {
   switch (v->id) {
-    case 5: case 11: return local ? 1.35 : 1.0;  // FP32, 16 x 8, two blocks per SM
+    case 5: case 11: return queue ? 2.1 : local ? 1.35 : 1.0;  // FP32, 16 x 8, two blocks per SM
     case 15: return 0.82;  // FP64 with FMA, non-ideal, 16 x 4 with 256 threads (13: 128)
     // FP32, non-ideal, 16 x 4 (14: 16 x 8): 0.63 measured; set so that it takes only patches of at most four
     // rows, where the count of fallback cells, each tile's halo included, is the other's
@@ -743,10 +745,10 @@ double tile_cost(const KernelVariant *v, bool local) {
     case 1: return 0.65;   // FP64, 8 x 8
     case 3: return 0.58;   // FP64 with FMA, 8 x 8
     case 4: return 1.22;   // FP64 with FMA, 16 x 12
-    case 6: return local ? 1.81 : 1.34;  // FP32, 16 x 8, one block per SM
+    case 6: return queue ? 2.1 : local ? 1.81 : 1.34;  // FP32, 16 x 8, one block per SM
     case 7: return 1.73;   // FP32, 32 x 8
     case 8: return 1.89;   // FP32, 16 x 16
-    case 21: return 1.90;  // FP32, 24 x 8 (alone 1.52; its own launch beside the other sizes' costs more)
+    case 21: return queue ? 1.52 : 1.90;  // FP32, 24 x 8 (alone 1.52; its own launch beside the other sizes' costs more)
     case 22: return 1.73;  // FP32 HLLD, 32 x 8
     default: return 1.0;   // 16 x 8 (non-ideal FP64: 16 x 4)
   }
@@ -1137,7 +1139,7 @@ extern "C" int dsp_create(const dsp_patch_desc *patches, int32_t npatch, const d
     for (int q = 0; q < kNumVariants; q++) {
       const KernelVariant *v = kVariants[q]();
       if (v->precision != prm->precision || v->riemann != prm->riemann || v->nonideal != nonideal) continue;
-      const double cost = tile_cost(v, prm->time_mode == 1) * ((cls_n[k][0] + v->tx - 1) / v->tx) * ((cls_n[k][1] + v->ty - 1) / v->ty);
+      const double cost = tile_cost(v, prm->time_mode == 1, prm->dispatcher == 0) * ((cls_n[k][0] + v->tx - 1) / v->tx) * ((cls_n[k][1] + v->ty - 1) / v->ty);
       if (cost < best && (v == var || fits(k, v))) {
         best = cost;
         varc[k] = v;
