@@ -677,7 +677,9 @@ __device__ __forceinline__ void march_tile(const DevCtx &c, const int P, const d
       }
     }
     // loads of plane p+2, of plane p+1 of the ring and of the old values to
-    // update: used after the next barrier
+    // update: used after the next barrier.  (FP32: they overwrite the updated
+    // cell that signal_new has just read.)
+    if constexpr (M::SL) cp_async_after_reads();
     const bool upd = it >= 2 && it <= nt_;
     const long long orow = (long long)(p - 1) * ny + y;
     int hm = 0, rm = 0, hes = 0, res = 0, ee = -1;  // blended values on their way

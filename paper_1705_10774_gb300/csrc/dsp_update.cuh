@@ -101,9 +101,12 @@ enum { GATHER_NOW = 0, GATHER_ISSUE = 1, GATHER_BLEND = 2 };
 template <int M>
 using GatherMode = std::integral_constant<int, M>;
 
-// (No memory clobber: what a copy writes is read only after cp_async_wait,
-// which has one; with it, each copy kept the next one's table lookups and
-// addresses from starting.)
+// (No memory clobber: with it, each copy kept the next one's table lookups
+// and addresses from starting.  What a copy writes is read only after
+// cp_async_wait, which has one.  What the place held before may have been read
+// by any thread before the last barrier, or by this thread before
+// cp_async_after_reads: nothing else keeps the compiler from moving a plain
+// read past the copy that overwrites it.)
 template <typename T>
 __device__ __forceinline__ void cp_async_elem(T *dst, const T *src) {
   static_assert(sizeof(T) == 4 || sizeof(T) == 8, "4- or 8-byte elements");
@@ -117,6 +120,8 @@ __device__ __forceinline__ void cp_async_if(float *dst, const float *src, bool o
   asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %2, 0;\n\t@p cp.async.ca.shared.global [%0], [%1], 4;\n\t}" ::"r"(d),
                "l"(src), "r"((int)on));
 }
+// Earlier plain accesses of this thread stay before the copies that follow.
+__device__ __forceinline__ void cp_async_after_reads() { asm volatile("" ::: "memory"); }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() {
