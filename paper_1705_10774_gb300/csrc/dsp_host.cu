@@ -446,7 +446,6 @@ __global__ void __launch_bounds__(256) smax_kernel(DevCtx c, int slot, int first
   const long long nc = (long long)nx * ny * nz;
   const T *bxa = base + 5 * nc, *bya = bxa + (long long)(nx + 1) * ny * nz, *bza = bya + (long long)nx * (ny + 1) * nz;
   const T gamma = (T)c.gamma;
-  const float gamma32 = (float)c.gamma;
   const bool bounds = sizeof(T) == 8 && !(c.eta > 0.0 || c.gad > 0.0);
   __shared__ int s_least;
   __shared__ double red[8];
@@ -473,7 +472,7 @@ __global__ void __launch_bounds__(256) smax_kernel(DevCtx c, int slot, int first
     if constexpr (sizeof(T) == 8) {
       if (bounds) {
         float above = 0.f, below = 0.f;
-        if (in) fast::signal_bounds(U, f[0], f[1], f[2], f[3], f[4], f[5], gamma32, above, below);
+        if (in) fast::signal_bounds(U, f[0], f[1], f[2], f[3], f[4], f[5], c.gamma32, c.gm132, above, below);
         const int w = __reduce_max_sync(0xffffffffu, __float_as_int(fmaxf(below, 0.f)));
         const int least = max(w, *(volatile int *)&s_least);
         if ((threadIdx.x & 31) == 0 && w == least) atomicMax(&s_least, w);
@@ -1206,6 +1205,8 @@ extern "C" int dsp_create(const dsp_patch_desc *patches, int32_t npatch, const d
       d.binv[l][k] = 1.0f / (float)bsz[l][k];
     }
   d.gamma = prm->gamma;
+  d.gamma32 = (float)prm->gamma;
+  d.gm132 = (float)(prm->gamma - 1.0);
   d.cfl = prm->cfl;
   d.dx = dx;
   d.dt_max = prm->dt_max;

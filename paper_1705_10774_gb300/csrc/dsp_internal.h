@@ -83,6 +83,7 @@ struct DevCtx {
   const long long *coff;   // [4][np+1] offsets of each patch in the caller's U, bx, by, bz arrays
   int *work_off;           // [np+1] first work item of each ready patch (prefix of tiles)
   double gamma, cfl, dx, dt_max;
+  float gamma32, gm132;    // gamma and gamma - 1, each rounded once to FP32
   // non-ideal MHD (Sec. 4.3): Ohmic resistivity, ambipolar drift coefficient
   // and ion density, Courant-like factors of their step limits (0 = off)
   double eta, gad, rhoi, cohm, cad;

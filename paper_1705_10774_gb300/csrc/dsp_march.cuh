@@ -124,7 +124,6 @@ __device__ __forceinline__ void march_tile(const DevCtx &c, const int P, const d
   const int lev = gp.level;
   const double dxl = ldexp(c.dx, -lev);
   T hdt = (T)(0.5 * dt / dxl), dtdx = (T)(dt / dxl);
-  const float gamma32 = (float)c.gamma;
   keep(gamma);
   keep(igm1);
   keep(gm1);
@@ -645,7 +644,7 @@ __device__ __forceinline__ void march_tile(const DevCtx &c, const int P, const d
 #pragma unroll
           for (int k = 0; k < 5; k++) un[k] = s0p[M::q(M::QU + k)];
           fast::signal_bounds(un, s0p[M::q(M::QNB)], s0p[M::q(M::QNB) + 1], s0p[M::q(M::QNB + 1)],
-                              s0p[M::q(M::QNB + 1) + PITCH], nfzl, nfzh, gamma32, above, below);
+                              s0p[M::q(M::QNB + 1) + PITCH], nfzl, nfzh, c.gamma32, c.gm132, above, below);
         }
         const int most = __reduce_max_sync(0xffffffffu, __float_as_int(fmaxf(below, 0.f)));
         if ((tid & 31) == 0 && most > S.least) atomicMax(&S.least, most);

@@ -1068,7 +1068,7 @@ __device__ __forceinline__ void process_tile(const DevCtx &c, const int P, const
         if (eval) {
           const int h = H1(ui, uj);
           fast::signal_bounds(unew, NBX[h], NBX[H1(ui + 1, uj)], NBY[h], NBY[H1(ui, uj + 1)], NBZp[h], NBZc[h],
-                              (float)gamma, above, below);
+                              c.gamma32, c.gm132, above, below);
           // the non-ideal step limits as signal speeds, each to a few roundings
           float ni = c.eta > 0.0 ? ohm32 : 0.f;
           if (c.gad > 0.0) {
