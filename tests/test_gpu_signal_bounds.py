@@ -4,12 +4,17 @@ Patches of two kinds of cell, a hot gas at rest and a dense stream whose
 speeds differ by a part in 1e5 to a fifth, in units and at ratios of specific
 heats where FP32 is short of range or of digits: the speeds are the oracle's,
 bit for bit."""
+import ctypes
+import os
+import subprocess
+
 import numpy as np
 import pytest
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
+from paper_1705_10774_gb300 import build as B
 from paper_1705_10774_gb300 import ics
 from paper_1705_10774_gb300.dispatch import Dispatch
 from oracle import Oracle
@@ -72,3 +77,95 @@ def test_units_of_large_and_small_velocities(scale, b):
     gas's speed came out up to 28 % low, and finite."""
     lay, state = _two_kinds(5.0 / 3.0, scale, (b, b, b))
     _same_speeds(lay, state, 5.0 / 3.0)
+
+
+# ------------------------------------------------------- the bounds themselves
+
+SRC = r"""
+#include "dsp_fast.cuh"
+__global__ void kernel(const double *in, int n, double gamma, float *above, float *below) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  double U[5];
+  for (int k = 0; k < 5; k++) U[k] = in[(long long)k * n + i];
+  const double *f = in + 5ll * n + i;
+  dsp::fast::signal_bounds(U, f[0], f[n], f[2ll * n], f[3ll * n], f[4ll * n], f[5ll * n], (float)gamma, (float)(gamma - 1.0),
+                           above[i], below[i]);
+}
+extern "C" int run(const double *in, int n, double gamma, float *above, float *below) {
+  kernel<<<(n + 255) / 256, 256>>>(in, n, gamma, above, below);
+  return (int)cudaDeviceSynchronize();
+}
+"""
+GAMMA = 5.0 / 3.0
+N = 1 << 18
+
+
+@pytest.fixture(scope="module")
+def bounds(tmp_path_factory):
+    """(above, below) of FP64 cells: signal_bounds, compiled by itself."""
+    d = tmp_path_factory.mktemp("bounds")
+    (d / "b.cu").write_text(SRC)
+    subprocess.check_call([B._nvcc(), "-O3", "-std=c++17", *B.ARCH, "-fmad=false", "-shared", "-Xcompiler", "-fPIC", "-I", B.CSRC,
+                           "-I", os.path.join(B.ROOT, "include"), str(d / "b.cu"), "-o", str(d / "b.so")])
+    lib = ctypes.CDLL(str(d / "b.so"))
+
+    def call(U, faces, gamma):
+        a = torch.from_numpy(np.stack([*U, *faces])).cuda()
+        out = torch.empty((2, a.shape[1]), dtype=torch.float32, device="cuda")
+        torch.cuda.synchronize()
+        P = ctypes.c_void_p
+        assert lib.run(P(a.data_ptr()), a.shape[1], ctypes.c_double(gamma), P(out[0].data_ptr()), P(out[1].data_ptr())) == 0
+        return out.cpu().numpy().astype(np.float64)
+
+    return call
+
+
+def _cells(rho, v, p, faces, gamma=GAMMA):
+    b2 = sum((0.5 * (faces[2 * k] + faces[2 * k + 1])) ** 2 for k in range(3))
+    return [rho, *(rho * x for x in v), p / (gamma - 1) + 0.5 * rho * sum(x * x for x in v) + 0.5 * b2], faces
+
+
+def _true(U, faces, gamma=GAMMA):
+    """The speeds of the same cells, p from the conserved values as the kernels take it."""
+    v, b = [m / U[0] for m in U[1:4]], [0.5 * (faces[2 * k] + faces[2 * k + 1]) for k in range(3)]
+    p = (gamma - 1) * (U[4] - 0.5 * U[0] * sum(x * x for x in v) - 0.5 * sum(x * x for x in b))
+    return _sum(gamma, U[0], np.maximum(p, 1e-20 * U[0]), b, v)
+
+
+def _hold(bounds, U, faces, gamma=GAMMA, some=0.5):
+    above, below = bounds(U, faces, gamma)
+    t = _true(U, faces, gamma)
+    assert np.all(above >= t) and np.all(~(below > t))
+    # and they are of use: within 1e-4 wherever the pressure is not lost in E
+    tight = (above <= 1.0001 * t) & (below >= 0.999 * t)
+    assert tight.mean() >= some
+
+
+def _draw(seed):
+    r = np.random.default_rng(seed)
+    return r, np.exp(r.normal(size=N)), r.normal(size=(3, N)), np.exp(2 * r.normal(size=N)), r.normal(size=(3, N))
+
+
+@pytest.mark.parametrize("kind", ["sound speed near the Alfven speed", "nearly along an axis"])
+def test_bounds_hold_where_the_discriminant_cancels(bounds, kind):
+    """s^2 - 4 a^2 b^2 loses half its digits for a field along an axis with
+    equal sound and Alfven speeds: the fast speed was off by 3e-4."""
+    r, rho, v, p, _ = _draw(1)
+    near = np.abs(1 + np.exp(r.uniform(np.log(1e-9), 0, N)) * r.choice([-1, 1], N))
+    along = near * np.sqrt(GAMMA * p)
+    across = 0 * p if kind.startswith("sound") else np.sqrt(p) * np.exp(r.uniform(np.log(1e-9), np.log(1e-2), N))
+    for axis in range(3):
+        f = [0 * p] * 6
+        f[2 * axis] = f[2 * axis + 1] = along
+        f[(2 * axis + 2) % 6] = f[(2 * axis + 3) % 6] = across
+        _hold(bounds, *_cells(rho, 0 * v, p, f))
+
+
+@pytest.mark.parametrize("gamma", [5.0 / 3.0, 1.4, 1.0001, 1.000001])
+@pytest.mark.parametrize("scale", [1e-7, 1e-3, 1.0, 1e5, 1e10, 1e13])
+def test_bounds_hold_across_units(bounds, scale, gamma):
+    _, rho, v, p, b = _draw(2)
+    _hold(bounds, *_cells(rho, scale * v, scale ** 2 * p, [scale * x for x in b for _ in range(2)], gamma), gamma)
+    for r in (1e-24, 1e-12, 1e12, 1e24):  # densities
+        _hold(bounds, *_cells(r * rho, 1e2 * v, 1e4 * r * p, [1e2 * np.sqrt(r) * x for x in b for _ in range(2)], gamma), gamma)
