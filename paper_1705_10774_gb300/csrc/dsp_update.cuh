@@ -1073,7 +1073,7 @@ __device__ __forceinline__ void process_tile(const DevCtx &c, const int P, const
           float ni = c.eta > 0.0 ? ohm32 : 0.f;
           if (c.gad > 0.0) {
             auto mean2 = [](double l, double r) {
-              const float b = 0.5f * (fast::trunc32(l) + fast::trunc32(r));
+              const float b = 0.5f * fast::trunc32(l + r);
               return b * b;
             };
             ni = fmaxf(ni, amb32 * (mean2(NBX[h], NBX[H1(ui + 1, uj)]) + mean2(NBY[h], NBY[H1(ui, uj + 1)]) + mean2(NBZp[h], NBZc[h])) /

@@ -169,3 +169,14 @@ def test_bounds_hold_across_units(bounds, scale, gamma):
     _hold(bounds, *_cells(rho, scale * v, scale ** 2 * p, [scale * x for x in b for _ in range(2)], gamma), gamma)
     for r in (1e-24, 1e-12, 1e12, 1e24):  # densities
         _hold(bounds, *_cells(r * rho, 1e2 * v, 1e4 * r * p, [1e2 * np.sqrt(r) * x for x in b for _ in range(2)], gamma), gamma)
+
+
+def test_bounds_hold_between_opposite_faces(bounds):
+    """A cell's field is the mean of its faces; the difference of two FP32
+    faces of opposite sign has the faces' error, not its own."""
+    r, rho, v, p, b = _draw(3)
+    f = []
+    for x in b:
+        big = np.exp(r.uniform(0, np.log(1e9), N))
+        f += [x - big, x + big]
+    _hold(bounds, *_cells(rho, v, p, f))
