@@ -1070,18 +1070,26 @@ __device__ __forceinline__ void process_tile(const DevCtx &c, const int P, const
           fast::signal_bounds(unew, NBX[h], NBX[H1(ui + 1, uj)], NBY[h], NBY[H1(ui, uj + 1)], NBZp[h], NBZc[h],
                               c.gamma32, c.gm132, above, below);
           // the non-ideal step limits as signal speeds, each to a few roundings
-          float ni = c.eta > 0.0 ? ohm32 : 0.f;
+          // (k B first: B^2 times the coefficient may be beyond FP32 where
+          // the limit is not); a cell whose limit FP32 cannot tell is
+          // evaluated, and bounds no other
+          const float ohm = c.eta > 0.0 ? ohm32 : 0.f;
+          float amb = 0.f;
           if (c.gad > 0.0) {
-            auto mean2 = [](double l, double r) {
+            const float k = amb32 / fast::trunc32(unew[0]);
+            auto part = [&](double l, double r) {
               const float b = 0.5f * fast::trunc32(l + r);
-              return b * b;
+              return (k * b) * b;
             };
-            ni = fmaxf(ni, amb32 * (mean2(NBX[h], NBX[H1(ui + 1, uj)]) + mean2(NBY[h], NBY[H1(ui, uj + 1)]) + mean2(NBZp[h], NBZc[h])) /
-                               fast::trunc32(unew[0]));
+            amb = part(NBX[h], NBX[H1(ui + 1, uj)]) + part(NBY[h], NBY[H1(ui, uj + 1)]) + part(NBZp[h], NBZc[h]);
           }
-          if (!(ni < 1e18f)) above = __int_as_float(0x7f800000);
-          above = fmaxf(above, ni * 1.00002f);
-          if (below > 0.f) below = fmaxf(below, ni * 0.99998f);
+          if (ohm < 1e18f && amb < 1e18f) {
+            const float ni = fmaxf(ohm, amb);
+            above = fmaxf(above, ni * 1.00002f);
+            if (below > 0.f) below = fmaxf(below, ni * 0.99998f);
+          } else {
+            above = __int_as_float(0x7f800000);
+          }
         }
         const int w = __reduce_max_sync(0xffffffffu, __float_as_int(fmaxf(below, 0.f)));
         const int least = max(w, *(volatile int *)&S.least);

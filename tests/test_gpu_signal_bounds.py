@@ -180,3 +180,30 @@ def test_bounds_hold_between_opposite_faces(bounds):
         big = np.exp(r.uniform(0, np.log(1e9), N))
         f += [x - big, x + big]
     _hold(bounds, *_cells(rho, v, p, f))
+
+
+def test_ambipolar_limit_beyond_fp32():
+    """The step limit of the ambipolar term as a speed, B^2 / rho times a
+    coefficient: B^2 times it overflows FP32 in the dense rows, whose limit is a
+    tenth of the thin ones'."""
+    lay = ics.cartesian((2, 1, 1), (16, 8, 4))
+    X, Y, Z = lay.base_cells
+    odd = np.broadcast_to(np.arange(Y)[:, None] % 2 == 1, (Z, Y, X))
+    one = np.ones((Z, Y, X))
+    f = ics.Fields(rho=np.where(odd, 1e24, 1e22), v=np.zeros((3, Z, Y, X)), p=1e20 * one, bx=np.where(odd, 3e9, 1e9),
+                   by=0 * one, bz=0 * one, gamma=GAMMA)
+    state = ics.to_patches(lay, f)
+    kw = dict(gamma=GAMMA, cfl=0.4, base_cells=lay.base_cells, box_len=lay.box_len, time_mode=0, rho_i=1.0,
+              gamma_ad=0.4 / (0.1 * 1e20 * lay.dx))
+    o = Oracle(lay.n, lay.lo, **kw)
+    o.set_state(*state)
+    o.advance(max_sweeps=1)
+    ref = o.get_times()[2]
+    assert np.all(ref > 1e15)
+    for precision in (0, 2):
+        g = Dispatch(lay.n, lay.lo, precision=precision, **kw)
+        g.set_state(*state)
+        g.advance(max_sweeps=1)
+        speed = g.pack(np.arange(lay.npatch), device=False)[1][:, 2]
+        g.close()
+        assert np.max(np.abs(speed / ref - 1)) <= (0 if precision == 0 else 1e-11)
