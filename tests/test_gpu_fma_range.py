@@ -8,6 +8,7 @@ pytestmark = pytest.mark.gpu
 
 from paper_1705_10774_gb300 import ics
 from paper_1705_10774_gb300.dispatch import Dispatch
+from oracle import Oracle
 
 GAMMA = 5.0 / 3.0
 
@@ -34,3 +35,26 @@ def test_densities_and_pressures_of_any_size(kw):
         g.close()
         first = first or out
         assert all(np.array_equal(a, b) for a, b in zip(out, first)), k
+
+
+def test_slopes_below_the_normal_range():
+    """Momenta of 1e-307 in a uniform gas at rest: the limited slopes are
+    rounded like any others (the tolerance of the parity tests)."""
+    lay = ics.cartesian((2, 1, 1), (17, 9, 6))
+    X, Y, Z = lay.base_cells
+    rng = np.random.default_rng(6)
+    one = np.ones((Z, Y, X))
+    f = ics.Fields(rho=one, v=1e-307 * rng.standard_normal((3, Z, Y, X)), p=0.6 * one, bx=0 * one, by=0 * one, bz=0 * one,
+                   gamma=GAMMA)
+    state = ics.to_patches(lay, f)
+    kw = dict(gamma=GAMMA, cfl=0.4, base_cells=lay.base_cells, box_len=lay.box_len, time_mode=0)
+    o = Oracle(lay.n, lay.lo, **kw)
+    o.set_state(*state)
+    o.advance(max_sweeps=1)
+    g = Dispatch(lay.n, lay.lo, precision=2, **kw)
+    g.set_state(*state)
+    g.advance(max_sweeps=1)
+    c = int(np.prod(lay.n[0]))
+    a, b = (np.asarray(s.get_state()[0]).reshape(lay.npatch, 5, c)[:, 1:4] for s in (g, o))
+    g.close()
+    assert np.max(np.abs(b)) < 1e-306 and np.max(np.abs(a - b)) <= 1e-11 * np.max(np.abs(b))
