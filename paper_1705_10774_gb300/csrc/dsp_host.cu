@@ -721,6 +721,26 @@ const KernelVariant *(*const kVariants[])() = {DSP_VARIANT_LIST(DSP_VARIANT_ENTR
 #undef DSP_VARIANT_ENTRY
 constexpr int kNumVariants = sizeof(kVariants) / sizeof(kVariants[0]);
 
+// The variant of a requested id; NULL if none has it.
+const KernelVariant *variant_of(int id) {
+  for (int k = 0; k < kNumVariants; k++)
+    if (kVariants[k]()->id == id) return kVariants[k]();
+#ifndef DSP_BOUNDS_CHECK
+#define DSP_VARIANT_ALIAS(ID, OF)                         \
+  if (id == ID) {                                         \
+    static const KernelVariant alias = [] {               \
+      KernelVariant v = *variant_##OF();                  \
+      v.id = ID;                                          \
+      return v;                                           \
+    }();                                                  \
+    return &alias;                                        \
+  }
+  DSP_VARIANT_ALIASES(DSP_VARIANT_ALIAS)
+#undef DSP_VARIANT_ALIAS
+#endif
+  return nullptr;
+}
+
 // SM time of one plane of one tile of a variant, relative to the other
 // variants of its form (measured on 256^3 cells in 32^3 patches: time of a
 // sweep over its tiles).  A patch's default variant is the one with the
@@ -741,14 +761,14 @@ double tile_cost(const KernelVariant *v, bool local, bool queue) {
     // rows, where the count of fallback cells, each tile's halo included, is the other's
     case 16: return 0.67;
     case 17: return 0.84;  // FP64, non-ideal, 16 x 4 with 256 threads (12: 128)
-    case 1: return 0.65;   // FP64, 8 x 8
-    case 3: return 0.58;   // FP64 with FMA, 8 x 8
-    case 4: return 1.22;   // FP64 with FMA, 16 x 12
     case 6: return queue ? 2.1 : local ? 1.81 : 1.34;  // FP32, 16 x 8, one block per SM
     case 7: return 1.73;   // FP32, 32 x 8
     case 8: return 1.89;   // FP32, 16 x 16
     case 21: return queue ? 1.52 : 1.90;  // FP32, 24 x 8 (alone 1.52; its own launch beside the other sizes' costs more)
     case 22: return 1.73;  // FP32 HLLD, 32 x 8
+    case 23: return 0.65;  // FP64, 8 x 8
+    case 24: return 0.58;  // FP64 with FMA, 8 x 8
+    case 25: return 1.22;  // FP64 with FMA, 16 x 12
     default: return 1.0;   // 16 x 8 (non-ideal FP64: 16 x 4)
   }
 }
@@ -1085,11 +1105,16 @@ extern "C" int dsp_create(const dsp_patch_desc *patches, int32_t npatch, const d
           gmap0[(size_t)((bz * mapd[0][1] + by) * mapd[0][0] + bx)] = -1;
   }
   // the update-kernel variant: the requested one, else the first of this precision
+  auto of_form = [&](const KernelVariant *v) {
+    return v && v->precision == prm->precision && v->riemann == prm->riemann && v->nonideal == nonideal;
+  };
   const KernelVariant *var = nullptr;
-  for (int k = 0; k < kNumVariants; k++) {
-    const KernelVariant *v = kVariants[k]();
-    if (v->precision != prm->precision || v->riemann != prm->riemann || v->nonideal != nonideal) continue;
-    if (prm->variant >= 0 ? v->id == prm->variant : !var) var = v;
+  if (prm->variant >= 0) {
+    const KernelVariant *v = variant_of(prm->variant);
+    if (of_form(v)) var = v;
+  } else {
+    for (int k = 0; k < kNumVariants && !var; k++)
+      if (of_form(kVariants[k]())) var = kVariants[k]();
   }
   if (!var) return DSP_ERR_INVALID_ARG;
   // size classes: one per distinct patch size (sweep dispatcher, at most
@@ -1137,7 +1162,7 @@ extern "C" int dsp_create(const dsp_patch_desc *patches, int32_t npatch, const d
     double best = INFINITY;
     for (int q = 0; q < kNumVariants; q++) {
       const KernelVariant *v = kVariants[q]();
-      if (v->precision != prm->precision || v->riemann != prm->riemann || v->nonideal != nonideal) continue;
+      if (!of_form(v)) continue;
       const double cost = tile_cost(v, prm->time_mode == 1, prm->dispatcher == 0) * ((cls_n[k][0] + v->tx - 1) / v->tx) * ((cls_n[k][1] + v->ty - 1) / v->ty);
       if (cost < best && (v == var || fits(k, v))) {
         best = cost;
