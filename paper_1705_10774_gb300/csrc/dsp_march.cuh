@@ -89,8 +89,13 @@ struct March {
   static constexpr int QB = SL ? QRAW + 5 : 77;  // [2] x- and y-faces of the plane to come
   static constexpr int NQ1 = !SL ? 80 : SZP ? 98 : 90;
   // tiles that have an SM to themselves: the second slice's values of a column
-  // blended in time, copied like the first's
+  // blended in time, copied like the first's (the bounds-checked build: in its
+  // one FP32 tile, so that these copies' addresses are tested too)
+#ifdef DSP_BOUNDS_CHECK
+  static constexpr bool DB = SL;
+#else
   static constexpr bool DB = SL && (PAIR ? NQ1 / 2 : NQ1) * PLANE * sizeof(T) > 110000;
+#endif
   static constexpr int QRB = NQ1;  // [8] (a ring column's: its places from QXR + 11 on)
   static constexpr int NQ = NQ1 + (DB ? 8 : 0);
   static constexpr int total = (PAIR ? NQ / 2 : NQ) * PLANE;
