@@ -112,12 +112,6 @@ __device__ __forceinline__ int pick_slices(const DevCtx &c, int Q, double t, Sli
   return DSP_OK;
 }
 
-// Local Courant step of patch P at time t (all FP64): the signal speed is the
-// largest over P's newest slice and every neighbour slice its guard fill
-// reads; the step is the power of two not above C dx / s (dx of P's level),
-// capped by dt_max,
-// halved until it divides t, and clipped to t_end.
-
 // The signal speeds of the slices of neighbour N that supply time t join M.
 template <bool CONC>
 __device__ __forceinline__ int guard_speed(const DevCtx &c, int N, double t, double &M) {
@@ -126,7 +120,10 @@ __device__ __forceinline__ int guard_speed(const DevCtx &c, int N, double t, dou
   for (int q = 0; q < pk.n; q++) M = fmax(M, slot_smax<CONC>(c, (long long)N * c.ns + pk.s[q]));
   return DSP_OK;
 }
-// The step of P at time t for the largest signal speed M.
+// Local Courant step of patch P at time t (all FP64) for M, the largest signal
+// speed of P's newest slice and of every neighbour slice its guard fill reads:
+// the power of two not above C dx / M (dx of P's level), capped by dt_max,
+// halved until it divides t, and clipped to t_end.
 __device__ __forceinline__ int step_of(const DevCtx &c, int P, double t, double t_end, double M, double *out) {
   const double dtc = c.cfl * ldexp(c.dx, -c.geo[P].level) / M;
   int e;
@@ -142,11 +139,11 @@ __device__ __forceinline__ int step_of(const DevCtx &c, int P, double t, double 
   *out = dt;
   return DSP_OK;
 }
-template <bool CONC>
-__device__ int patch_dt(const DevCtx &c, int P, double t, double t_end, double *out) {
-  double M = slot_smax<CONC>(c, (long long)P * c.ns + newest<CONC>(c, P));
+// The step of P at time t, by one thread of the ready queue.
+__device__ __forceinline__ int patch_dt(const DevCtx &c, int P, double t, double t_end, double *out) {
+  double M = slot_smax<true>(c, (long long)P * c.ns + newest<true>(c, P));
   for (int k = c.nbl_off[P]; k < c.nbl_off[P + 1]; k++) {
-    const int rc = guard_speed<CONC>(c, c.nbl[k], t, M);
+    const int rc = guard_speed<true>(c, c.nbl[k], t, M);
     if (rc != DSP_OK) return rc;
   }
   return step_of(c, P, t, t_end, M, out);
@@ -176,18 +173,19 @@ __device__ bool slot_free(const DevCtx &c, int P) {
 
 // Eq. (1): P is ready when t_P < t_end and t_P <= t_N + g dt_N for every
 // neighbour N (dt_N its last step, 0 before the first), and, with g > 0,
-// its oldest slice is free.  Writes t_P.
+// its oldest slice is free.  The condition on one neighbour:
 template <bool CONC>
+__device__ __forceinline__ bool not_ahead(const DevCtx &c, double t, int N) {
+  return t <= slot_time<CONC>(c, (long long)N * c.ns + newest<CONC>(c, N)) + c.grace * c.dt_last[N];
+}
+// All of it, by one thread of the ready queue.  Writes t_P.
 __device__ __forceinline__ bool is_ready(const DevCtx &c, int P, double t_end, double *tP) {
-  const int ns = c.ns;
-  const double t = slot_time<CONC>(c, (long long)P * ns + newest<CONC>(c, P));
+  const double t = slot_time<true>(c, (long long)P * c.ns + newest<true>(c, P));
   *tP = t;
   if (!(t < t_end)) return false;
-  for (int k = c.nbl_off[P]; k < c.nbl_off[P + 1]; k++) {
-    const int N = c.nbl[k];
-    if (!(t <= slot_time<CONC>(c, (long long)N * ns + newest<CONC>(c, N)) + c.grace * c.dt_last[N])) return false;
-  }
-  if (c.grace > 0.0 && !slot_free<CONC>(c, P)) return false;
+  for (int k = c.nbl_off[P]; k < c.nbl_off[P + 1]; k++)
+    if (!not_ahead<true>(c, t, c.nbl[k])) return false;
+  if (c.grace > 0.0 && !slot_free<true>(c, P)) return false;
   return true;
 }
 

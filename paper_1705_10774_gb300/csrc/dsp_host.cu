@@ -172,10 +172,8 @@ __device__ void ready_part(const DevCtx &c, int P, double t_end) {
     if (lane == 0) c.ctl[CTL_NOTDONE] = 1;
     const int k0 = c.nbl_off[P], k1 = c.nbl_off[P + 1];
     bool ok = true;
-    for (int k = k0 + lane; k < k1; k += 32) {
-      const int N = c.nbl[k];
-      if (!(t <= slot_time<false>(c, (long long)N * ns + newest<false>(c, N)) + c.grace * c.dt_last[N])) ok = false;
-    }
+    for (int k = k0 + lane; k < k1; k += 32)
+      if (!not_ahead<false>(c, t, c.nbl[k])) ok = false;
     ok = __all_sync(0xffffffffu, ok);
     if (ok && c.grace > 0.0) ok = slot_free<false>(c, P);
     if (ok) {
@@ -238,8 +236,9 @@ __device__ __forceinline__ int block_scan_flag(int flag, int *s_wsum, int &s_tot
 // and done / deadlock.
 //
 // FUSED (contexts of at most FUSE_MAX patches): parts 1 and 2 in the same
-// block and launch; with so few patches a sweep is three launches too many
-// long, not three too few wide.
+// block and launch.  With so few patches each part is done sooner than the next
+// kernel starts (64 sweeps of ten patches, loading and reading included: 13.7 ms
+// with three launches a sweep, 13.4 with one).
 constexpr int FUSE_MAX = 128;
 template <bool FUSED>
 __global__ void __launch_bounds__(PLAN_NT) plan_compact_kernel(DevCtx c, double t_end, int global_mode, int publish_only) {
@@ -315,9 +314,10 @@ __global__ void __launch_bounds__(PLAN_NT) plan_compact_kernel(DevCtx c, double 
   if (tid == 0) c.ctl[CTL_CLS + c.ncls] = s_kb;
   // Planes per work item.  A sweep whose tiles leave blocks idle (a few
   // patches, or one large one) cuts each z run into m equal parts: a part of
-  // s planes costs s + 2 (its halo planes), and the sweep takes as many
-  // rounds of blocks as the items need, so the m that minimises rounds x
-  // (s + 5/2) is taken (half a plane for an item's start).  Eight patches of
+  // s planes computes slopes and fluxes on s + 2 (a halo plane at either end)
+  // and fills its pipeline first, which counts as half a plane; the sweep takes
+  // as many rounds of blocks as the items need, so the m that minimises rounds
+  // x (s + 5/2) is taken.  Eight patches of
   // 16^3 (16 tiles), FP64 without FMA: 1.43 ms a sweep uncut, 0.32 ms cut; ten
   // of 30 x 4 x 4 (20 tiles): 0.43 and 0.21 ms.  Sweeps that fill the GPU
   // four times over are left whole.

@@ -221,14 +221,14 @@ __device__ __forceinline__ int owner_table(const DevCtx &c, int P, int lev, doub
 
 namespace dsp {
 
-// Advance one tile of patch P by dt (all threads of the block take part).
-// On return the tile's new cells, faces and signal speed are written.  CONC:
-// other blocks publish patch times concurrently (ready-queue dispatcher).
-// RS: Riemann solver of the face fluxes (0 HLL, 1 HLLD).  NI: add the
-// non-ideal Ohmic and ambipolar EMFs (DISPATCH I, Sec. 4.3) and their
-// Poynting flux; these variants gather each plane synchronously (no copies
-// in flight) and hold three planes of faces.
-template <typename T, int TX, int TY, int NT, bool CONC, int RS, int NI>
+// Advance one tile of patch P by dt with the non-ideal Ohmic and ambipolar
+// EMFs (DISPATCH I, Sec. 4.3) and their Poynting flux (all threads of the
+// block take part).  On return the tile's new cells, faces and signal speed
+// are written.  CONC: other blocks publish patch times concurrently
+// (ready-queue dispatcher); planes are then gathered synchronously, by sweeps
+// with copies in flight.  RS: Riemann solver of the face fluxes (0 HLL, 1
+// HLLD).
+template <typename T, int TX, int TY, int NT, bool CONC, int RS>
 __device__ __forceinline__ void process_tile(const DevCtx &c, const int P, const double dt, const int tile,
                                              const int zlo, const int zrun, T *sm, TileShared<T, NT> &S) {
   static_assert(TX * TY <= NT, "one updated cell per thread");
@@ -939,13 +939,10 @@ __device__ __forceinline__ void process_tile(const DevCtx &c, const int P, const
         const T apz = pmax0(SZ[H1N + hm], SZ[H1N + h0]), amz = nmax0(SZ[hm], SZ[h0]);
         const T apa = d == 0 ? ap2 : apz, ama = d == 0 ? am2 : amz;
         const T apb = d == 0 ? apz : ap2, amb = d == 0 ? amz : am2;
-        T e = emf_of(Ell, Erl, Elr, E0, Ba_ll, Ba_rl, Ba_lr, ba0, Bb_ll, Bb_rl, Bb_lr, bb0, apa, ama, apb, amb);
-        if constexpr (NI != 0) {
-          const T en = d == 0 ? eni_x(i, j, p) : eni_y(i, j, p);
-          (d == 0 ? ENX : ENY)[par * H1N + h0] = en;
-          e = e + en;
-        }
-        (d == 0 ? EXc : EYc)[h0] = e;
+        const T e = emf_of(Ell, Erl, Elr, E0, Ba_ll, Ba_rl, Ba_lr, ba0, Bb_ll, Bb_rl, Bb_lr, bb0, apa, ama, apb, amb);
+        const T en = d == 0 ? eni_x(i, j, p) : eni_y(i, j, p);
+        (d == 0 ? ENX : ENY)[par * H1N + h0] = en;
+        (d == 0 ? EXc : EYc)[h0] = e + en;
       };
       if constexpr (POOL) {
         constexpr int DU0 = (NE + 31) / 32 * 32;
@@ -960,13 +957,11 @@ __device__ __forceinline__ void process_tile(const DevCtx &c, const int P, const
         if (div)
           for (int ci = tid; ci < TX * TY; ci += NT) div_item(ci);
       }
-      {
-        if (div) {
-          for (int ci = tid; ci < (TX + 1) * (TY + 1); ci += NT) {
-            const int i = ci % (TX + 1), j = ci / (TX + 1), h = H1(i, j);
-            if (i <= tx && j < ty) FXE[par * H1N + h] = FX[4 * H1N + h];
-            if (i < tx && j <= ty) FYE[par * H1N + h] = FY[4 * H1N + h];
-          }
+      if (div) {
+        for (int ci = tid; ci < (TX + 1) * (TY + 1); ci += NT) {
+          const int i = ci % (TX + 1), j = ci / (TX + 1), h = H1(i, j);
+          if (i <= tx && j < ty) FXE[par * H1N + h] = FX[4 * H1N + h];
+          if (i < tx && j <= ty) FYE[par * H1N + h] = FY[4 * H1N + h];
         }
       }
     }
@@ -977,46 +972,44 @@ __device__ __forceinline__ void process_tile(const DevCtx &c, const int P, const
     // energy divergence is formed from its x- and y-faces' ideal fluxes plus
     // theirs (edge EMFs averaged to the face, cell-centred B averaged over
     // the two cells of the face)
-    if constexpr (NI != 0) {
-      if (it >= 1) {
-        // z-faces (i, j, p-1/2): d = z, a = x, b = y
-        for (int ci = tid; ci < TX * TY; ci += NT) {
-          const int i = ci % TX, j = ci / TX;
-          if (i >= tx || j >= ty) continue;
-          const int h = H1(i, j);
-          const T Ea = half * (ENX[par * H1N + h] + ENX[par * H1N + H1(i, j + 1)]);
-          const T Eb = half * (ENY[par * H1N + h] + ENY[par * H1N + H1(i + 1, j)]);
-          const T Ba = half * (wc(BX, i, j, p - 1) + wc(BX, i, j, p));
-          const T Bb = half * (wc(BY, i, j, p - 1) + wc(BY, i, j, p));
-          FZc[4 * H1N + h] = FZc[4 * H1N + h] + (Ea * Bb - Eb * Ba);
-        }
+    if (it >= 1) {
+      // z-faces (i, j, p-1/2): d = z, a = x, b = y
+      for (int ci = tid; ci < TX * TY; ci += NT) {
+        const int i = ci % TX, j = ci / TX;
+        if (i >= tx || j >= ty) continue;
+        const int h = H1(i, j);
+        const T Ea = half * (ENX[par * H1N + h] + ENX[par * H1N + H1(i, j + 1)]);
+        const T Eb = half * (ENY[par * H1N + h] + ENY[par * H1N + H1(i + 1, j)]);
+        const T Ba = half * (wc(BX, i, j, p - 1) + wc(BX, i, j, p));
+        const T Bb = half * (wc(BY, i, j, p - 1) + wc(BY, i, j, p));
+        FZc[4 * H1N + h] = FZc[4 * H1N + h] + (Ea * Bb - Eb * Ba);
       }
-      if (it >= 2) {
-        const int q = p - 1, pr = par ^ 1;
-        // x-face (i-1/2, j, q): d = x, a = y (levels q-1/2, q+1/2), b = z
-        auto ftx = [&](int i, int j) -> T {
-          const T Ea = half * (ENY[pr * H1N + H1(i, j)] + ENY[par * H1N + H1(i, j)]);
-          const T Eb = half * (ENZ[H1(i, j)] + ENZ[H1(i, j + 1)]);
-          const T Ba = half * (wc(BY, i - 1, j, q) + wc(BY, i, j, q));
-          const T Bb = half * (wc(BZ, i - 1, j, q) + wc(BZ, i, j, q));
-          return FXE[pr * H1N + H1(i, j)] + (Ea * Bb - Eb * Ba);
-        };
-        // y-face (i, j-1/2, q): d = y, a = z, b = x (levels q-1/2, q+1/2)
-        auto fty = [&](int i, int j) -> T {
-          const T Ea = half * (ENZ[H1(i, j)] + ENZ[H1(i + 1, j)]);
-          const T Eb = half * (ENX[pr * H1N + H1(i, j)] + ENX[par * H1N + H1(i, j)]);
-          const T Ba = half * (wc(BZ, i, j - 1, q) + wc(BZ, i, j, q));
-          const T Bb = half * (wc(BX, i, j - 1, q) + wc(BX, i, j, q));
-          return FYE[pr * H1N + H1(i, j)] + (Ea * Bb - Eb * Ba);
-        };
-        for (int ci = tid; ci < TX * TY; ci += NT) {
-          const int i = ci % TX, j = ci / TX;
-          if (i >= tx || j >= ty) continue;
-          DUp[4 * H1N + H1(i, j)] = (ftx(i + 1, j) - ftx(i, j)) + (fty(i, j + 1) - fty(i, j));
-        }
-      }
-      __syncthreads();
     }
+    if (it >= 2) {
+      const int q = p - 1, pr = par ^ 1;
+      // x-face (i-1/2, j, q): d = x, a = y (levels q-1/2, q+1/2), b = z
+      auto ftx = [&](int i, int j) -> T {
+        const T Ea = half * (ENY[pr * H1N + H1(i, j)] + ENY[par * H1N + H1(i, j)]);
+        const T Eb = half * (ENZ[H1(i, j)] + ENZ[H1(i, j + 1)]);
+        const T Ba = half * (wc(BY, i - 1, j, q) + wc(BY, i, j, q));
+        const T Bb = half * (wc(BZ, i - 1, j, q) + wc(BZ, i, j, q));
+        return FXE[pr * H1N + H1(i, j)] + (Ea * Bb - Eb * Ba);
+      };
+      // y-face (i, j-1/2, q): d = y, a = z, b = x (levels q-1/2, q+1/2)
+      auto fty = [&](int i, int j) -> T {
+        const T Ea = half * (ENZ[H1(i, j)] + ENZ[H1(i + 1, j)]);
+        const T Eb = half * (ENX[pr * H1N + H1(i, j)] + ENX[par * H1N + H1(i, j)]);
+        const T Ba = half * (wc(BZ, i, j - 1, q) + wc(BZ, i, j, q));
+        const T Bb = half * (wc(BX, i, j - 1, q) + wc(BX, i, j, q));
+        return FYE[pr * H1N + H1(i, j)] + (Ea * Bb - Eb * Ba);
+      };
+      for (int ci = tid; ci < TX * TY; ci += NT) {
+        const int i = ci % TX, j = ci / TX;
+        if (i >= tx || j >= ty) continue;
+        DUp[4 * H1N + H1(i, j)] = (ftx(i + 1, j) - ftx(i, j)) + (fty(i, j + 1) - fty(i, j));
+      }
+    }
+    __syncthreads();
 
     // ---- E: update plane p-1 and the z-faces at p-1/2
     const bool upd = it >= 2;
@@ -1153,13 +1146,10 @@ __device__ __forceinline__ void process_tile(const DevCtx &c, const int P, const
         const T ama = nmax0(SXc[hrl], SXc[hrr]);
         const T apb = pmax0(SYc[H1N + hlr], SYc[H1N + hrr]);
         const T amb = nmax0(SYc[hlr], SYc[hrr]);
-        T ez = emf_of(Ell, Erl, Elr, Err, ll_bx, rl_bx, lr_bx, rr_bx, ll_by, rl_by, lr_by, rr_by, apa, ama, apb, amb);
-        if constexpr (NI != 0) {
-          const T en = eni_z(i, j, p);
-          ENZ[hrr] = en;
-          ez = ez + en;
-        }
-        EZ[hrr] = ez;
+        const T ez = emf_of(Ell, Erl, Elr, Err, ll_bx, rl_bx, lr_bx, rr_bx, ll_by, rl_by, lr_by, rr_by, apa, ama, apb, amb);
+        const T en = eni_z(i, j, p);
+        ENZ[hrr] = en;
+        EZ[hrr] = ez + en;
       };
       auto carry_item = [&](int c) {
         const int i = c % (TX + 2) - 1, j = c / (TX + 2) - 1, h = H1(i, j);
@@ -1244,7 +1234,7 @@ __device__ __forceinline__ void process_tile(const DevCtx &c, const int P, const
 template <typename T, int TX, int TY, int NT, bool CONC, int RS, int NI>
 __device__ __forceinline__ void update_tile(const DevCtx &c, int P, double dt, int tile, int zlo, int zrun, T *sm,
                                             TileShared<T, NT> &S) {
-  if constexpr (NI != 0) process_tile<T, TX, TY, NT, CONC, RS, NI>(c, P, dt, tile, zlo, zrun, sm, S);
+  if constexpr (NI != 0) process_tile<T, TX, TY, NT, CONC, RS>(c, P, dt, tile, zlo, zrun, sm, S);
   else march_tile<T, TX, TY, NT, CONC, RS>(c, P, dt, tile, zlo, zrun, sm, S);
 }
 // its shared memory in bytes
@@ -1320,12 +1310,12 @@ static __device__ void try_queue(const DevCtx &c, int Q, double t_end) {
   for (int attempt = 0; attempt < 8; attempt++) {
     if (ld_acquire(&c.p_state[Q]) != 0) return;
     double tq;
-    if (!is_ready<true>(c, Q, t_end, &tq)) return;
+    if (!is_ready(c, Q, t_end, &tq)) return;
     if (atomicCAS(&c.p_state[Q], 0, 1) != 0) return;
     __threadfence();
-    if (is_ready<true>(c, Q, t_end, &tq)) {
+    if (is_ready(c, Q, t_end, &tq)) {
       double dt;
-      const int rc = patch_dt<true>(c, Q, tq, t_end, &dt);
+      const int rc = patch_dt(c, Q, tq, t_end, &dt);
       if (rc != DSP_OK) {
         set_error(c, rc, Q, -1);
         return;
