@@ -62,9 +62,9 @@ NONIDEAL = dict(eta=1e-4, gamma_ad=75.0, rho_i=1.0)
 # of one launch divided by the cells it updated (captures of smaller cases
 # of the same kernel: traffic grows in proportion to the cells); a variant
 # without an entry reports null.
-TRAFFIC_PER_CELL = {25: (549.944064e6 + 449.829888e6) / 7077888, 7: (241.673728e6 + 193.319424e6) / 7077888,
-                    10: (567.815936e6 + 445.036032e6) / 7077888, 14: (235.899648e6 + 193.474048e6) / 7077888,
-                    15: (526.316800e6 + 424.240640e6) / 7077888, 22: (242.319104e6 + 194.282752e6) / 7077888}
+TRAFFIC_PER_CELL = {25: (550.531840e6 + 450.511104e6) / 7077888, 7: (241.881600e6 + 193.002496e6) / 7077888,
+                    10: (565.389568e6 + 445.015808e6) / 7077888, 14: (235.899648e6 + 193.474048e6) / 7077888,
+                    15: (526.330880e6 + 423.851776e6) / 7077888, 22: (242.319104e6 + 194.282752e6) / 7077888}
 
 
 def guard_fraction(n, g):

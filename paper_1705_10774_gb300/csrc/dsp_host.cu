@@ -767,8 +767,8 @@ double tile_cost(const KernelVariant *v, bool local, bool queue) {
     case 21: return queue ? 1.52 : 1.90;  // FP32, 24 x 8 (alone 1.52; its own launch beside the other sizes' costs more)
     case 22: return 1.73;  // FP32 HLLD, 32 x 8
     case 23: return 0.65;  // FP64, 8 x 8
-    case 24: return 0.58;  // FP64 with FMA, 8 x 8
-    case 25: return 1.22;  // FP64 with FMA, 16 x 12
+    case 24: return 0.60;  // FP64 with FMA, 8 x 8
+    case 25: return 1.21;  // FP64 with FMA, 16 x 12
     default: return 1.0;   // 16 x 8 (non-ideal FP64: 16 x 4)
   }
 }

@@ -28,9 +28,9 @@
 // slots and the latency of a column's chains, so a thread's positions are
 // fixed for the whole tile and every shared address is one base plus a
 // constant.  Measured, 256^3 in 32^3 patches, a sweep: FP64 with FMA 50.7 ms
-// for the block marching phase by phase over shared planes, 36.2 so (76 % of
-// the FP64 pipe's slots, where 84 % can be had; 926 FP64 operations a cell
-// instead of 1530; 79 GB/s of algorithmic traffic); without FMA 78.3 and 67.7;
+// for the block marching phase by phase over shared planes, 36.4 so (76 % of
+// the FP64 pipe's slots, where 84 % can be had; 930 FP64 operations a cell
+// instead of 1530; 79 GB/s of algorithmic traffic); without FMA 78.3 and 68.1;
 // FP32 4.33 and 2.53 (84 instead of 166 warp instructions a cell, 47 % of the
 // issue slots, 567 GB/s).
 #pragma once

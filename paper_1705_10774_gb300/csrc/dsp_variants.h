@@ -7,9 +7,9 @@
 // (0 HLL, 1 HLLD), non-ideal terms (1: the Ohmic and ambipolar EMFs).
 // Ideal MHD has a thread per column of the tile and its halo, so the tile
 // sets the block; wide tiles have less halo per cell (512^3 cells in 32^3
-// patches, a sweep: FP64 with FMA 278 ms for 16 x 12, 317 for 16 x 8, 366 for
-// 8 x 8; FP32 20.5 ms for 32 x 8, 21.8 for 16 x 16, 25.5 for two blocks of
-// 16 x 8, 32.1 for one, 38.3 for 24 x 8, which 32^3 does not fit), small ones fit
+// patches, a sweep: FP64 with FMA 282 ms for 16 x 12, 323 for 16 x 8, 382 for
+// 8 x 8; FP32 20.5 ms for 32 x 8, 22.2 for 16 x 16, 25.8 for two blocks of
+// 16 x 8, 32.1 for one, 38.4 for 24 x 8, which 32^3 does not fit), small ones fit
 // small patches.  The registers of a column (255 in FP64, 168 in FP32) set how
 // many warps an SM holds.  The non-ideal tiles hold four planes of faces in
 // shared memory, so the FP64 rows use a smaller one.  All variants of one
